@@ -420,8 +420,8 @@ int pmk_measure_imad_peak(pmk_ctx *ctx, double *mad_lo_per_clk_per_sm, double *s
  *          with b primes (nbits/64 for an ordinary key).
  *   tpi:   lanes of a warp that hold one exponentiation (a power of two
  *          dividing 32 and the limb count); 0 restores the built-in default.
- *   form:  Montgomery product form, 0 = one add-with-carry chain per lane and
- *          row, 1 = independent 64-bit column accumulators.
+ *   form:  0, or 1 where pmk_list_kernel_configs lists it; both name the same
+ *          kernel (1 was a second Montgomery product form).
  * Returns EUNSUPPORTED if that geometry is not compiled in.  Results are
  * bit-identical for every geometry; only speed differs.
  */

@@ -12,31 +12,28 @@ struct BlindEntry {
   size_t smem;
 };
 
-template <int S, int TPI, int FORM, int NT = dev::kThreads>
+template <int S, int TPI, int NT = dev::kThreads>
 BlindEntry make_blind() {
-  return BlindEntry{S, TPI, NT, reinterpret_cast<const void *>(&dev::k_blind_crt<S, TPI, FORM, NT>),
+  return BlindEntry{S, TPI, NT, reinterpret_cast<const void *>(&dev::k_blind_crt<S, TPI, NT>),
                     dev::modexp_smem_bytes<S>(TPI, NT)};
 }
 
 // Throughput geometries (the CRT defaults), then geometries with more lanes
 // per instance for small batches (a shorter chain per exponentiation).
 const BlindEntry *blind_entries(int *count) {
-  using dev::kChain;
-  using dev::kCols;
   static const BlindEntry entries[] = {
-      make_blind<2, 2, kChain>(),  make_blind<4, 2, kChain>(),  make_blind<8, 2, kChain>(),
-      make_blind<16, 2, kChain>(), make_blind<32, 4, kCols, 64>(), make_blind<48, 8, kChain>(),
-      make_blind<64, 8, kChain>(), make_blind<96, 8, kChain>(),  make_blind<128, 16, kChain>(),
+      make_blind<2, 2>(),  make_blind<4, 2>(),  make_blind<8, 2>(),
+      make_blind<16, 2>(), make_blind<32, 4, 64>(), make_blind<48, 8>(),
+      make_blind<64, 8>(), make_blind<96, 8>(),  make_blind<128, 16>(),
   };
   *count = (int)(sizeof(entries) / sizeof(entries[0]));
   return entries;
 }
 
 const BlindEntry *blind_entries_latency(int *count) {
-  using dev::kChain;
   static const BlindEntry entries[] = {
-      make_blind<16, 8, kChain>(),  make_blind<32, 16, kChain>(), make_blind<48, 16, kChain>(),
-      make_blind<64, 32, kChain>(), make_blind<96, 16, kChain>(), make_blind<128, 32, kChain>(),
+      make_blind<16, 8>(),  make_blind<32, 16>(), make_blind<48, 16>(),
+      make_blind<64, 32>(), make_blind<96, 16>(), make_blind<128, 32>(),
   };
   *count = (int)(sizeof(entries) / sizeof(entries[0]));
   return entries;

@@ -338,7 +338,7 @@ std::vector<ModexpEntry> entries(bool crt) {
 const ModexpEntry *find_exact(uint32_t limbs, KernelConfig cfg, bool crt) {
   static const std::vector<ModexpEntry> full = entries(false), residue = entries(true);
   for (const ModexpEntry &e : crt ? residue : full)
-    if (e.limbs == (int)limbs && e.tpi == (int)cfg.tpi && e.form == (int)cfg.form && e.table == cfg.table) return &e;
+    if (e.limbs == (int)limbs && e.tpi == (int)cfg.tpi && cfg.form < 2 && (e.forms >> cfg.form & 1u) && e.table == cfg.table) return &e;
   return nullptr;
 }
 
@@ -520,9 +520,8 @@ uint32_t crt_sum_block_instances(uint32_t limbs) {
   return 0u;
 }
 
-// Defaults measured on GB300 (1 MiB and 100 MiB workloads at 2048 bits):
-// 64-limb full-width and 32-limb CRT residues run fastest with independent
-// columns at 8 and 4 lanes; other widths use the carry-chain form.
+// Throughput defaults, measured on GB300 (1 MiB and 100 MiB workloads at 2048
+// bits).  The form only names the geometry (see ModexpEntry::forms).
 KernelConfig default_config(uint32_t limbs, bool crt) {
   KernelConfig c;
   switch (limbs) {
@@ -539,17 +538,13 @@ KernelConfig default_config(uint32_t limbs, bool crt) {
 
 int list_configs(uint32_t limbs, bool crt, KernelConfig *out, int max) {
   int k = 0;
-  const std::vector<ModexpEntry> all = entries(crt);
-  for (size_t i = 0; i < all.size(); i++) {
-    const ModexpEntry &e = all[i];
-    if (e.limbs != (int)limbs || e.table != kTableFull) continue;  // geometries; small-table twins are not listed
-    bool seen = false;  // block-size twins are one geometry
-    for (size_t j = 0; j < i && !seen; j++)
-      seen = all[j].limbs == e.limbs && all[j].tpi == e.tpi && all[j].form == e.form && all[j].table == kTableFull;
-    if (seen) continue;
-    if (k < max && out) out[k] = KernelConfig{(uint32_t)e.tpi, (uint32_t)e.form};
-    k++;
-  }
+  for (uint32_t form = 0; form < 2; form++)
+    for (const ModexpEntry &e : entries(crt)) {
+      // geometries; small-table twins are not listed
+      if (e.limbs != (int)limbs || e.table != kTableFull || !(e.forms >> form & 1u)) continue;
+      if (k < max && out) out[k] = KernelConfig{(uint32_t)e.tpi, form};
+      k++;
+    }
   return k;
 }
 
@@ -611,8 +606,7 @@ int launch_modexp(ExpMode mode, uint32_t limbs, KernelConfig cfg, const KeyDev *
   if (!groups && (unsigned long long)K * (crt ? parts : 1) > 65535ull) return PMK_EINVAL;  // grid.y
   const ModexpEntry *e = find_entry(limbs, cfg, crt);
   if (!e) return PMK_EUNSUPPORTED;
-  const void *fn = groups ? e->fn_grp : e->fn;
-  const int rc = configure_smem(fn, e->smem);
+  const int rc = configure_smem(e->fn, e->smem);
   if (rc != PMK_OK) return rc;
   const long long per_key = ((long long)n + K - 1) / K;
   const int ipb = e->threads / e->tpi;
@@ -625,7 +619,7 @@ int launch_modexp(ExpMode mode, uint32_t limbs, KernelConfig cfg, const KeyDev *
   int np = crt ? (int)parts : 1;
   void *args[] = {(void *)&keys, (void *)&K,   (void *)&in, (void *)&out,
                   (void *)&nl,   (void *)&sel, (void *)&np, (void *)&groups};
-  return cuda_rc(cudaLaunchKernel(fn, grid, dim3(e->threads), args, e->smem, st));
+  return cuda_rc(cudaLaunchKernel(e->fn, grid, dim3(e->threads), args, e->smem, st));
 }
 
 }  // namespace pmk

@@ -22,7 +22,7 @@ static_assert(kTableMax >= 16, "the joint tables use rows 0-7 (A) and 8-15 (B)")
 // and B (Montgomery form, this instance); tbl gets A's odd powers in rows
 // 0..maxa and B's in rows 8..8+maxb; ybuf is the squaring buffer.  sched is
 // a Schedule2 (block-uniform).
-template <int S, int TPI, int FORM>
+template <int S, int TPI>
 __device__ __forceinline__ void exp2_window(uint32_t (&a)[S / TPI], uint32_t *tbl, uint32_t *ybuf,
                                             const uint32_t *__restrict__ sched, uint32_t nsteps, uint32_t maxa,
                                             uint32_t maxb, const uint32_t (&nn)[S / TPI], uint32_t n0, uint32_t r) {
@@ -37,14 +37,14 @@ __device__ __forceinline__ void exp2_window(uint32_t (&a)[S / TPI], uint32_t *tb
     __syncwarp();
     store_slice<L>(ybuf, a, r);
     __syncwarp();
-    mont<S, TPI, FORM>(a, ybuf, nn, n0, r);  // X^2
+    mont<S, TPI>(a, ybuf, nn, n0, r);  // X^2
     __syncwarp();
     store_slice<L>(ybuf, a, r);
     load_slice<L>(a, base, r);
     __syncwarp();
 #pragma unroll 1
     for (uint32_t k = 1; k <= maxi; k++) {  // row k = X^(2k+1)
-      mont<S, TPI, FORM>(a, ybuf, nn, n0, r);
+      mont<S, TPI>(a, ybuf, nn, n0, r);
       store_slice<L>(base + k * ROW, a, r);
     }
     __syncwarp();
@@ -54,7 +54,7 @@ __device__ __forceinline__ void exp2_window(uint32_t (&a)[S / TPI], uint32_t *tb
   const uint32_t ia0 = (s0 >> 8) & 0xffu, ib0 = s0 & 0xffu;
   if (ia0 != 0xffu) {
     load_slice<L>(a, tbl + ia0 * ROW, r);
-    if (ib0 != 0xffu) mont<S, TPI, FORM>(a, tbl + (8 + ib0) * ROW, nn, n0, r);
+    if (ib0 != 0xffu) mont<S, TPI>(a, tbl + (8 + ib0) * ROW, nn, n0, r);
   } else {
     load_slice<L>(a, tbl + (8 + ib0) * ROW, r);
   }
@@ -67,10 +67,10 @@ __device__ __forceinline__ void exp2_window(uint32_t (&a)[S / TPI], uint32_t *tb
       __syncwarp();
       store_slice<L>(ybuf, a, r);
       __syncwarp();
-      mont<S, TPI, FORM>(a, ybuf, nn, n0, r);
+      mont<S, TPI>(a, ybuf, nn, n0, r);
     }
-    if (ia != 0xffu) mont<S, TPI, FORM>(a, tbl + ia * ROW, nn, n0, r);
-    if (ib != 0xffu) mont<S, TPI, FORM>(a, tbl + (8 + ib) * ROW, nn, n0, r);
+    if (ia != 0xffu) mont<S, TPI>(a, tbl + ia * ROW, nn, n0, r);
+    if (ib != 0xffu) mont<S, TPI>(a, tbl + (8 + ib) * ROW, nn, n0, r);
   }
 }
 
@@ -78,7 +78,7 @@ __device__ __forceinline__ void exp2_window(uint32_t (&a)[S / TPI], uint32_t *tb
 // of the chunk's key (grid as the CRT mode of k_modexp: blockIdx.y = key *
 // parts + i).  With `status`, a c_r divisible by r_i (no inverse mod N)
 // sets kStatusNotInvertible.
-template <int S, int TPI, int FORM, int NT>
+template <int S, int TPI, int NT>
 __global__ void __launch_bounds__(NT) k_blind_crt(const KeyDev *__restrict__ keys, uint32_t K,
                                                   const uint32_t *__restrict__ cstar, const uint32_t *__restrict__ cr,
                                                   uint32_t *__restrict__ out, long long n, int parts,
@@ -114,9 +114,9 @@ __global__ void __launch_bounds__(NT) k_blind_crt(const KeyDev *__restrict__ key
   const uint32_t n0 = kd.n0h[prime];
   uint32_t nn[L], a[L];
   load_slice_global<L>(nn, kd.P[prime], r);
-  crt_input<S, TPI, FORM>(a, cstar + t * W, active, parts, sR2, sR3, nn, n0, r);  // A = c* R mod r_i
+  crt_input<S, TPI>(a, cstar + t * W, active, parts, sR2, sR3, nn, n0, r);  // A = c* R mod r_i
   store_slice<L>(tbl, a, r);
-  crt_input<S, TPI, FORM>(a, cr + t * W, active, parts, sR2, sR3, nn, n0, r);     // B = c_r R mod r_i
+  crt_input<S, TPI>(a, cr + t * W, active, parts, sR2, sR3, nn, n0, r);     // B = c_r R mod r_i
   uint32_t any = 0;
 #pragma unroll
   for (int j = 0; j < L; j++) any |= a[j];
@@ -126,9 +126,9 @@ __global__ void __launch_bounds__(NT) k_blind_crt(const KeyDev *__restrict__ key
   }
   if (status && active && r == 0 && any == 0) report(status, kStatusNotInvertible, t);
   store_slice<L>(tbl + 8 * ROW, a, r);
-  exp2_window<S, TPI, FORM>(a, tbl, ybuf, kd.sched_blind[prime], kd.nsteps_blind[prime], kd.maxa_blind[prime],
+  exp2_window<S, TPI>(a, tbl, ybuf, kd.sched_blind[prime], kd.nsteps_blind[prime], kd.maxa_blind[prime],
                             kd.maxb_blind[prime], nn, n0, r);
-  mont<S, TPI, FORM>(a, sOne, nn, n0, r);  // leave the Montgomery domain
+  mont<S, TPI>(a, sOne, nn, n0, r);  // leave the Montgomery domain
   if (active) {
     uint32_t *o = out + t * W + prime * S + r * L;
 #pragma unroll

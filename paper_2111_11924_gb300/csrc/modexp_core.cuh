@@ -10,18 +10,17 @@
 // (< N).  Exponentiation is Algorithm 2's square-and-multiply generalised to a
 // left-to-right sliding window of odd powers (schedules built on the host).
 //
-// Cost model on this GPU (measured with row-shaped loops, one multiplier per
-// row and the multiplicands in registers): mad.lo issues at up to 64
-// lanes/clk/SM but the high half of a 32x32 product at only about 22, and a
-// wide multiply (both halves, with or without a 64-bit addend) at 16-24
-// depending on the warps per SM.  The high half is therefore the cost of a
-// MAC whatever form it takes.  Integer adds issue on the ALU pipe, in
-// parallel.  So each row forms its L products with wide multiplies and folds
-// them in with two add-with-carry chains (low halves at word j, high halves
-// at word j + 1).
-// Lane-to-lane carries are deferred: a lane keeps a small pending word above
-// its L limbs, which the per-row shift moves into its own top limb; after the
-// last row a ballot carry-lookahead resolves them in O(1) warp operations.
+// Cost model on this GPU (measured with row-shaped loops, MAC per clock per SM
+// at 4 / 8 / 16 warps per SM): a wide multiply-add with carry in and out
+// (mad.lo.cc + madc.hi.cc of one 64-bit pair) 19 / 26 / 27, a wide multiply
+// whose halves are then added into 64-bit columns 16 / 20 / 20, mad.lo 58 /
+// 63 / 64.  The multiplier's high half bounds every form, and the adds are
+// free only inside the multiply-add, so a row is built of carry chains over
+// 64-bit pairs: one instruction per MAC and nothing but the chain ends on the
+// ALU pipe.
+// Lane-to-lane carries are deferred: a lane keeps small pending words above
+// its L limbs; after the last row a ballot carry-lookahead resolves them in
+// O(1) warp operations.
 #pragma once
 
 #include <cstdint>
@@ -70,55 +69,11 @@ struct Layout {
   static constexpr int kConstRows = 3;  // R^2, one, R^3
 };
 
-// Row forms: how one row t += a * y turns into instructions.
-//   kWide: L wide multiplies (64-bit products), low and high halves folded in
-//          by two add-with-carry chains on the integer ALU pipe;
-//   kMadc: mad.lo/mad.hi with carry in and out, so the multiply unit also
-//          does the additions (nothing on the ALU pipe but the chain ends).
-// A Montgomery row pair (a * y_i, then q * N) may use a different form for
-// each half, to balance the multiply and ALU pipes.
-enum RowForm : int { kWide = 0, kMadc = 1 };
-#ifndef PMK_ROW_FORM
-#define PMK_ROW_FORM 0
-#endif
-constexpr int kFormA = (PMK_ROW_FORM == 1 || PMK_ROW_FORM == 2) ? kMadc : kWide;  // a * y_i
-constexpr int kFormN = (PMK_ROW_FORM == 1 || PMK_ROW_FORM == 3) ? kMadc : kWide;  // q * N
-
-__device__ __forceinline__ void madlo_cc(uint32_t &t, uint32_t a, uint32_t y) {
-  asm volatile("mad.lo.cc.u32 %0, %1, %2, %0;" : "+r"(t) : "r"(a), "r"(y));
-}
-__device__ __forceinline__ void madclo_cc(uint32_t &t, uint32_t a, uint32_t y) {
-  asm volatile("madc.lo.cc.u32 %0, %1, %2, %0;" : "+r"(t) : "r"(a), "r"(y));
-}
-__device__ __forceinline__ void madhi_cc(uint32_t &t, uint32_t a, uint32_t y) {
-  asm volatile("mad.hi.cc.u32 %0, %1, %2, %0;" : "+r"(t) : "r"(a), "r"(y));
-}
-__device__ __forceinline__ void madchi_cc(uint32_t &t, uint32_t a, uint32_t y) {
-  asm volatile("madc.hi.cc.u32 %0, %1, %2, %0;" : "+r"(t) : "r"(a), "r"(y));
-}
-
 // (t, c0, c1) += a * y, where t is this lane's L limbs and (c0, c1) the
 // pending words above them.
-template <int L, int FORM>
+template <int L>
 __device__ __forceinline__ void row_mac(uint32_t (&t)[L], uint32_t &c0, uint32_t &c1, const uint32_t (&a)[L],
                                         uint32_t y) {
-  if constexpr (FORM == kMadc) {
-    madlo_cc(t[0], a[0], y);
-#pragma unroll
-    for (int j = 1; j < L; j++) madclo_cc(t[j], a[j], y);
-    addc_cc(c0, c0, 0u);
-    addc(c1, c1, 0u);
-    if constexpr (L > 1) {
-      madhi_cc(t[1], a[0], y);
-#pragma unroll
-      for (int j = 1; j < L - 1; j++) madchi_cc(t[j + 1], a[j], y);
-      madchi_cc(c0, a[L - 1], y);
-    } else {
-      madhi_cc(c0, a[0], y);
-    }
-    addc(c1, c1, 0u);
-    return;
-  }
   uint32_t lo[L], hi[L];
 #pragma unroll
   for (int j = 0; j < L; j++) {
@@ -207,15 +162,12 @@ __device__ __forceinline__ void finalize(uint32_t (&t)[L], uint32_t c0, const ui
   }
 }
 
-// Rows of a product processed per unrolled group (y limbs fetched as 16- or
-// 8-byte broadcasts).  In the carry-chain form a group of L rows (L = limbs
-// per lane, 6 to 16) brings the per-row shift of the lane's words back to
-// the starting registers, so no register moves remain: measured 3-18%
-// faster than groups of 4 at 6, 8, 12 and 16 limbs per lane.  The column
-// form measured no gain and keeps groups of 4.
-template <int S, int L, bool kChainForm>
+// Rows of a product per unrolled group.  A group of L rows (or 2 L, for whole
+// 16-byte reads of y) brings the per-row shift of the lane's words back to
+// the starting registers, so no register moves remain.
+template <int S, int L>
 __host__ __device__ constexpr int row_group() {
-  return (kChainForm && L >= 6 && L <= 16 && L % 2 == 0 && S % L == 0) ? L : (S % 4 == 0) ? 4 : 2;
+  return (L % 4 == 0) ? L : (L % 2 == 0 && S % (2 * L) == 0) ? 2 * L : (L % 2 == 0) ? L : (S % 4 == 0) ? 4 : 2;
 }
 
 template <int K>
@@ -237,11 +189,13 @@ __device__ __forceinline__ void load_y(uint32_t (&yv)[K], const uint32_t *ys) {
 
 // a <- MontMul(a, y) = a y R^-1 mod N.  a: this lane's limbs (any value < R);
 // ys: y's S limbs in shared memory (y < N), read as 16-byte broadcasts.
+// One row at a time, one add-with-carry chain per lane: the form for an odd
+// number of limbs per lane, which has no pairs.
 template <int S, int TPI>
 __device__ __forceinline__ void mont_mul(uint32_t (&a)[S / TPI], const uint32_t *ys, const uint32_t (&nn)[S / TPI],
                                          uint32_t n0, uint32_t r) {
   constexpr int L = S / TPI;
-  constexpr int kStep = row_group<S, L, true>();
+  constexpr int kStep = row_group<S, L>();
   uint32_t t[L];
 #pragma unroll
   for (int j = 0; j < L; j++) t[j] = 0;
@@ -252,10 +206,10 @@ __device__ __forceinline__ void mont_mul(uint32_t (&a)[S / TPI], const uint32_t 
     load_y<kStep>(yv, ys + i0);
 #pragma unroll
     for (int u = 0; u < kStep; u++) {
-      row_mac<L, kFormA>(t, c0, c1, a, yv[u]);
+      row_mac<L>(t, c0, c1, a, yv[u]);
       uint32_t q = t[0] * n0;
       if constexpr (TPI > 1) q = __shfl_sync(kFull, q, 0, TPI);
-      row_mac<L, kFormN>(t, c0, c1, nn, q);
+      row_mac<L>(t, c0, c1, nn, q);
       // T /= 2^32: limb 0 of lane 0 is now zero; every lane takes the next
       // lane's limb 0 as its new top limb and folds its pending word into it.
       uint32_t in = 0;
@@ -275,85 +229,147 @@ __device__ __forceinline__ void mont_mul(uint32_t (&a)[S / TPI], const uint32_t 
   for (int j = 0; j < L; j++) a[j] = t[j];
 }
 
-// a <- MontMul(a, y), column form.  Each lane keeps one 64-bit accumulator
-// per limb position ("column"): the low half of a product a_j * y_i goes to
-// column j and its high half to column j + 1, so a row is L independent
-// column updates instead of one add-with-carry chain through the lane.
-// Columns absorb at most four 32-bit terms per row and live at most S + L
-// rows, so they stay below 2^42.  The row shift moves a whole column (two
-// shuffles); column carries are propagated once, before finalize.
-template <int S, int TPI>
-__device__ __forceinline__ void mont_mul_cols(uint32_t (&a)[S / TPI], const uint32_t *ys, const uint32_t (&nn)[S / TPI],
-                                              uint32_t n0, uint32_t r) {
-  constexpr int L = S / TPI;
-  constexpr int kStep = row_group<S, L, false>();
-  uint64_t acc[L];
+// (lo, hi) += a y, a 64-bit pair, with the carry out (and in, for madc) in the
+// condition code; each compiles to one wide multiply-add.
+__device__ __forceinline__ void mad_wide_cc(uint32_t &lo, uint32_t &hi, uint32_t a, uint32_t y) {
+  asm volatile("mad.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.cc.u32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(y));
+}
+__device__ __forceinline__ void madc_wide_cc(uint32_t &lo, uint32_t &hi, uint32_t a, uint32_t y) {
+  asm volatile("madc.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.cc.u32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(y));
+}
+
+// (w[OFF + 2 i], w[OFF + 2 i + 1]) += m[PAR + 2 i] y for i < L / 2 in one
+// carry chain.  CIN: the chain takes the condition code's carry.  The carry
+// out is left in the condition code.
+template <int L, int PAR, int OFF, bool CIN, int W>
+__device__ __forceinline__ void pair_chain(uint32_t (&w)[W], const uint32_t (&m)[L], uint32_t y) {
+  if constexpr (CIN) {
+    madc_wide_cc(w[OFF], w[OFF + 1], m[PAR], y);
+  } else {
+    mad_wide_cc(w[OFF], w[OFF + 1], m[PAR], y);
+  }
 #pragma unroll
-  for (int j = 0; j < L; j++) acc[j] = 0;
+  for (int i = 1; i < L / 2; i++) madc_wide_cc(w[OFF + 2 * i], w[OFF + 2 * i + 1], m[PAR + 2 * i], y);
+}
+
+// a <- MontMul(a, y) for an even number of limbs per lane: two rows per step.
+//
+// The lane's part of T is kept as two sums of 64-bit pairs: e, whose word j
+// has weight 2^(32 j), and o, whose word j has weight 2^(32 (j + 1)).  The
+// even limbs times y_i and the odd limbs times y_{i+1} land on e's pairs, the
+// other two products on o's, so each of the four is one carry chain of L / 2
+// wide multiply-adds.  The quotient of both rows is one 64-bit value,
+// q = T (-N^-1) mod 2^64 of lane 0, and T /= 2^64 moves whole pairs: e and o
+// keep their roles and a step needs one broadcast of q and one shift between
+// lanes.  A chain's carry out is held back (c0, c1, c2: weights L, L + 1,
+// L + 2) and joins the words that the shift brings in.
+//
+// Bound: the wide multiply-add, 4 L per lane and step against about 26 other
+// instructions on other pipes.  Measured against the column form that it
+// replaces (2048-bit keys, full d): 12.76 vs 17.67 ms at 1 MiB, 104.9 vs
+// 142.7 ms at 10 MiB; CRT 3.41 vs 4.64 ms at 1 MiB.
+template <int S, int TPI>
+__device__ __forceinline__ void mont_mul_pairs(uint32_t (&a)[S / TPI], const uint32_t *ys,
+                                               const uint32_t (&nn)[S / TPI], uint32_t n0, uint32_t r) {
+  constexpr int L = S / TPI;
+  static_assert(L % 2 == 0, "pairs of limbs");
+  constexpr int kStep = row_group<S, L>();
+  // -N^-1 mod 2^64 from its low word by one Newton step (lane 0's is used).
+  const uint64_t n01 = ((uint64_t)nn[1] << 32) | nn[0];
+  const uint32_t k1 = (uint32_t)(((uint64_t)n0 * (2 + n01 * n0)) >> 32);
+  const uint32_t below_top = (r == TPI - 1) ? 0u : kFull;
+  uint32_t e[L + 2], o[L];
+#pragma unroll
+  for (int j = 0; j < L; j++) e[j] = o[j] = 0;
+  e[L] = e[L + 1] = 0;
+  uint32_t c0 = 0, c1 = 0, c2 = 0;
+  // The words of weight 0 and 1 go to the lane below (lane 0's are zero).
+  auto shifted_out = [&](uint32_t &x0, uint32_t &x1) {
+    x0 = e[0];
+    x1 = e[1] + o[0];
+    if constexpr (TPI > 1) {
+      x0 = __shfl_down_sync(kFull, x0, 1, TPI) & below_top;
+      x1 = __shfl_down_sync(kFull, x1, 1, TPI) & below_top;
+    } else {
+      x0 = x1 = 0;
+    }
+  };
 #pragma unroll 1
   for (int i0 = 0; i0 < S; i0 += kStep) {
     uint32_t yv[kStep];
     load_y<kStep>(yv, ys + i0);
 #pragma unroll
-    for (int u = 0; u < kStep; u++) {
-      uint32_t hprev = 0;
+    for (int u = 0; u < kStep; u += 2) {
+      // T /= 2^64.  o's first pair ends in weight 2; the carry of that sum has
+      // weight 3, the first word of the new o, where the next chain starts.
+      uint32_t x0, x1, drop;
+      shifted_out(x0, x1);
+      add_cc(drop, e[1], o[0]);
+      addc_cc(e[2], e[2], o[1]);
+      uint32_t f[L + 2], p[L];
 #pragma unroll
-      for (int j = 0; j < L; j++) {
-        const uint64_t p = (uint64_t)a[j] * yv[u];
-        acc[j] += (uint64_t)(uint32_t)p + hprev;
-        hprev = (uint32_t)(p >> 32);
-      }
-      uint64_t top = hprev;  // column L: the next lane's column 0 before the shift
-      uint32_t q = (uint32_t)acc[0] * n0;
-      if constexpr (TPI > 1) q = __shfl_sync(kFull, q, 0, TPI);
-      hprev = 0;
+      for (int j = 0; j < L; j++) f[j] = e[j + 2];
 #pragma unroll
-      for (int j = 0; j < L; j++) {
-        const uint64_t p = (uint64_t)nn[j] * q;
-        acc[j] += (uint64_t)(uint32_t)p + hprev;
-        hprev = (uint32_t)(p >> 32);
-      }
-      top += hprev;
-      // T /= 2^32: column 0 of lane 0 is now zero mod 2^32 and its high part
-      // carries into column 1; every other lane's column 0 moves down to the
-      // previous lane's top column.
-      uint64_t in = 0;
+      for (int j = 0; j < L - 2; j++) p[j] = o[j + 2];
+      p[L - 2] = p[L - 1] = 0;
+      pair_chain<L, 1, 0, true>(p, a, yv[u]);
+      uint32_t d1;
+      addc(d1, 0u, 0u);
+      add_cc(f[L - 2], f[L - 2], c0);
+      addc_cc(f[L - 1], f[L - 1], c1);
+      addc(c2, c2, 0u);
+      add_cc(f[L - 2], f[L - 2], x0);
+      addc_cc(f[L - 1], f[L - 1], x1);
+      addc(f[L], c2, 0u);
+      // T += a (y_i + 2^32 y_{i+1})
+      pair_chain<L, 0, 0, false>(f, a, yv[u]);
+      addc(f[L], f[L], 0u);
+      pair_chain<L, 0, 0, false>(p, a, yv[u + 1]);
+      addc(f[L + 1], d1, 0u);
+      uint32_t q0 = f[0] * n0;
+      uint32_t q1 = __umulhi(f[0], n0) + f[0] * k1 + (f[1] + p[0]) * n0;
       if constexpr (TPI > 1) {
-        const uint32_t lo = __shfl_down_sync(kFull, (uint32_t)acc[0], 1, TPI);
-        const uint32_t hi = __shfl_down_sync(kFull, (uint32_t)(acc[0] >> 32), 1, TPI);
-        if (r != TPI - 1) in = ((uint64_t)hi << 32) | lo;
+        q0 = __shfl_sync(kFull, q0, 0, TPI);
+        q1 = __shfl_sync(kFull, q1, 0, TPI);
       }
-      const uint64_t carry0 = (r == 0) ? (acc[0] >> 32) : 0;
+      pair_chain<L, 1, 2, false>(f, a, yv[u + 1]);
+      addc(c2, 0u, 0u);
+      // T += N (q_0 + 2^32 q_1)
+      pair_chain<L, 0, 0, false>(f, nn, q0);
+      addc(c0, 0u, 0u);
+      pair_chain<L, 1, 0, false>(p, nn, q0);
+      addc(c1, 0u, 0u);
+      pair_chain<L, 0, 0, false>(p, nn, q1);
+      addc(c1, c1, 0u);
+      pair_chain<L, 1, 2, false>(f, nn, q1);
+      addc(c2, c2, 0u);
 #pragma unroll
-      for (int j = 0; j < L - 1; j++) acc[j] = acc[j + 1];
-      acc[L - 1] = in + top;
-      acc[0] += carry0;
+      for (int j = 0; j < L + 2; j++) e[j] = f[j];
+#pragma unroll
+      for (int j = 0; j < L; j++) o[j] = p[j];
     }
   }
-  uint32_t t[L];
-  uint64_t c = 0;
+  // The last shift, then e and o in one carry chain.
+  uint32_t x0, x1, drop;
+  shifted_out(x0, x1);
+  add_cc(e[L], e[L], c0);
+  addc_cc(e[L + 1], e[L + 1], c1);
+  addc(c2, c2, 0u);
+  add_cc(e[L], e[L], x0);
+  addc_cc(e[L + 1], e[L + 1], x1);
+  addc(c2, c2, 0u);
+  add_cc(drop, e[1], o[0]);
 #pragma unroll
-  for (int j = 0; j < L; j++) {
-    const uint64_t v = acc[j] + c;
-    t[j] = (uint32_t)v;
-    c = v >> 32;
-  }
-  finalize<L, TPI>(t, (uint32_t)c, nn, r);
-#pragma unroll
-  for (int j = 0; j < L; j++) a[j] = t[j];
+  for (int j = 0; j < L; j++) addc_cc(a[j], e[j + 2], (j + 1 < L) ? o[j + 1] : 0u);
+  addc(c2, c2, 0u);
+  finalize<L, TPI>(a, c2, nn, r);
 }
 
-// Montgomery product forms: kChain = mont_mul (one add-with-carry chain per
-// lane and row), kCols = mont_mul_cols (independent 64-bit columns).  Which is
-// faster depends on limbs per lane and on how many warps a batch provides, so
-// each compiled geometry names its form.
-enum MontForm : int { kChain = 0, kCols = 1 };
-
-template <int S, int TPI, int FORM>
+template <int S, int TPI>
 __device__ __forceinline__ void mont(uint32_t (&a)[S / TPI], const uint32_t *ys, const uint32_t (&nn)[S / TPI],
                                      uint32_t n0, uint32_t r) {
-  if constexpr (FORM == kCols) {
-    mont_mul_cols<S, TPI>(a, ys, nn, n0, r);
+  if constexpr ((S / TPI) % 2 == 0) {
+    mont_mul_pairs<S, TPI>(a, ys, nn, n0, r);
   } else {
     mont_mul<S, TPI>(a, ys, nn, n0, r);
   }
@@ -418,7 +434,7 @@ __device__ __forceinline__ void load_slice_global(uint32_t (&a)[L], const uint32
 // table (at least maxidx + 1 rows: the table size the schedule was built
 // for), ybuf: one row of this instance.  sched: steps of make_schedule()
 // (block-uniform).
-template <int S, int TPI, int FORM>
+template <int S, int TPI>
 __device__ __forceinline__ void exp_window(uint32_t (&a)[S / TPI], uint32_t *tbl, uint32_t *ybuf,
                                            const uint32_t *__restrict__ sched, uint32_t nsteps, uint32_t maxidx,
                                            const uint32_t (&nn)[S / TPI], uint32_t n0, uint32_t r) {
@@ -428,14 +444,14 @@ __device__ __forceinline__ void exp_window(uint32_t (&a)[S / TPI], uint32_t *tbl
   if (maxidx > 0) {
     store_slice<L>(ybuf, a, r);
     __syncwarp();
-    mont<S, TPI, FORM>(a, ybuf, nn, n0, r);  // x^2
+    mont<S, TPI>(a, ybuf, nn, n0, r);  // x^2
     __syncwarp();
     store_slice<L>(ybuf, a, r);
     load_slice<L>(a, tbl, r);
     __syncwarp();
 #pragma unroll 1
     for (uint32_t k = 1; k <= maxidx; k++) {  // T[k] = T[k-1] x^2 = x^(2k+1)
-      mont<S, TPI, FORM>(a, ybuf, nn, n0, r);
+      mont<S, TPI>(a, ybuf, nn, n0, r);
       store_slice<L>(tbl + k * ROW, a, r);
     }
     __syncwarp();
@@ -450,9 +466,9 @@ __device__ __forceinline__ void exp_window(uint32_t (&a)[S / TPI], uint32_t *tbl
       __syncwarp();
       store_slice<L>(ybuf, a, r);
       __syncwarp();
-      mont<S, TPI, FORM>(a, ybuf, nn, n0, r);
+      mont<S, TPI>(a, ybuf, nn, n0, r);
     }
-    if (idx != 0xffu) mont<S, TPI, FORM>(a, tbl + idx * ROW, nn, n0, r);
+    if (idx != 0xffu) mont<S, TPI>(a, tbl + idx * ROW, nn, n0, r);
   }
 }
 

@@ -12,7 +12,7 @@ namespace dev {
 // from the top piece: MontMul(c_top, R^3) = c_top R^2 is the Montgomery form
 // of c_top R, MontMul(c_j, R^2) that of c_j, and MontMul(x, R^2) multiplies
 // the value in Montgomery form by R.  Two pieces take two products.
-template <int S, int TPI, int FORM>
+template <int S, int TPI>
 __device__ __forceinline__ void crt_input(uint32_t (&a)[S / TPI], const uint32_t *c, bool active, int parts,
                                           const uint32_t *sR2, const uint32_t *sR3, const uint32_t (&nn)[S / TPI],
                                           uint32_t n0, uint32_t r) {
@@ -25,18 +25,18 @@ __device__ __forceinline__ void crt_input(uint32_t (&a)[S / TPI], const uint32_t
 #pragma unroll
     for (int j = 0; j < L; j++) lo[j] = a[j] = 0;
   }
-  mont<S, TPI, FORM>(a, sR3, nn, n0, r);   // c_top R^2
-  mont<S, TPI, FORM>(lo, sR2, nn, n0, r);  // c_next R
+  mont<S, TPI>(a, sR3, nn, n0, r);   // c_top R^2
+  mont<S, TPI>(lo, sR2, nn, n0, r);  // c_next R
   mod_add<L, TPI>(a, lo, nn, r);           // (c_top R + c_next) R
   for (int piece = parts - 3; piece >= 0; piece--) {
-    mont<S, TPI, FORM>(a, sR2, nn, n0, r);  // value * R, still in Montgomery form
+    mont<S, TPI>(a, sR2, nn, n0, r);  // value * R, still in Montgomery form
     if (active) {
       load_slice_global<L>(lo, c + piece * S, r);
     } else {
 #pragma unroll
       for (int j = 0; j < L; j++) lo[j] = 0;
     }
-    mont<S, TPI, FORM>(lo, sR2, nn, n0, r);
+    mont<S, TPI>(lo, sR2, nn, n0, r);
     mod_add<L, TPI>(a, lo, nn, r);
   }
 }
@@ -98,19 +98,10 @@ __device__ __forceinline__ long long slot_chunk(const uint32_t *__restrict__ grp
 // NT threads per block (128, or 64 where smaller blocks fit more
 // instances in an SM's shared memory).  TABLE (kTableFull or kTableSmall)
 // sizes the odd-power tables in shared memory and selects the key's
-// schedules built for it.  MINB: the minimum resident blocks per SM declared
-// to ptxas (0: none); 1 lets it use more registers, which pays for one
-// geometry (see the CRT instantiations).  GRP = false: round robin only.
-// GRP = true: a key group table (grp, explicit key indices) when grp is
-// given, round robin when it is null.  Two instantiations because the table
-// lookup in the prologue, though outside the exponentiation, changes how
-// ptxas compiles the whole kernel: 38 instead of 32 registers at 64 limbs
-// and 32 lanes, round-robin launches up to 18% slower at 100 KB, and a few
-// column-form geometries 1-2% faster (measured); each geometry names the
-// instantiation that serves its round-robin launches (make_entry).
-template <int S, int TPI, bool CRT, int FORM, int NT = kThreads, int TABLE = kTableFull, int MINB = 0,
-          bool GRP = false>
-__global__ void __launch_bounds__(NT, MINB) k_modexp(const KeyDev *__restrict__ keys, uint32_t K,
+// schedules built for it.  grp: a key group table (explicit key indices), or
+// null for round robin.
+template <int S, int TPI, bool CRT, int NT = kThreads, int TABLE = kTableFull>
+__global__ void __launch_bounds__(NT) k_modexp(const KeyDev *__restrict__ keys, uint32_t K,
                                                const uint32_t *__restrict__ in, uint32_t *__restrict__ out,
                                                long long n, int sel, int parts, const uint32_t *__restrict__ grp) {
   constexpr int L = S / TPI;
@@ -125,21 +116,10 @@ __global__ void __launch_bounds__(NT, MINB) k_modexp(const KeyDev *__restrict__ 
   uint32_t *tbl = smem + Layout<S>::kConstRows * ROW + g * INST;
   uint32_t *ybuf = tbl + ROWS * ROW;
 
-  uint32_t key, prime;
-  long long first = 0;  // round robin: the block's first chunk
-  BlockChunks bc{};     // key groups: the block's key and first slot
-  if constexpr (GRP) {
-    prime = CRT ? (grp ? blockIdx.y : blockIdx.y % (uint32_t)parts) : 0;
-    bc = block_chunks(grp, K, n, IPB, CRT ? blockIdx.y / (uint32_t)parts : blockIdx.y);
-    if (!bc.any) return;  // block-uniform: no instance of this block has a chunk
-    key = bc.key;
-  } else {
-    key = CRT ? blockIdx.y / (uint32_t)parts : blockIdx.y;
-    prime = CRT ? blockIdx.y % (uint32_t)parts : 0;
-    first = key + (long long)blockIdx.x * IPB * K;
-    if (first >= n) return;  // block-uniform: no instance of this block has a chunk
-  }
-  const KeyDev &kd = keys[key];
+  const uint32_t prime = CRT ? (grp ? blockIdx.y : blockIdx.y % (uint32_t)parts) : 0;
+  const BlockChunks bc = block_chunks(grp, K, n, IPB, CRT ? blockIdx.y / (uint32_t)parts : blockIdx.y);
+  if (!bc.any) return;  // block-uniform: no instance of this block has a chunk
+  const KeyDev &kd = keys[bc.key];
   const uint32_t *M = CRT ? kd.P[prime] : kd.N;
   const uint32_t *R2 = CRT ? kd.R2h[prime] : kd.R2;
   const uint32_t *sched = CRT ? (sel ? kd.sched_hinv[TABLE][prime] : kd.sched_h[TABLE][prime])
@@ -159,17 +139,9 @@ __global__ void __launch_bounds__(NT, MINB) k_modexp(const KeyDev *__restrict__ 
   // After the barrier the warps are independent: a warp whose instances all
   // lie past the last chunk of the key leaves (chunks and slots of a key are
   // in order, padding last, so its first instance decides).
-  long long t;
-  bool active;
-  if constexpr (GRP) {
-    if (slot_chunk(grp, K, n, bc, (threadIdx.x / 32) * (32 / TPI)) < 0) return;
-    t = slot_chunk(grp, K, n, bc, g);
-    active = t >= 0;
-  } else {
-    if (first + (long long)((threadIdx.x / 32) * (32 / TPI)) * K >= n) return;
-    t = first + (long long)g * K;
-    active = t < n;
-  }
+  if (slot_chunk(grp, K, n, bc, (threadIdx.x / 32) * (32 / TPI)) < 0) return;
+  const long long t = slot_chunk(grp, K, n, bc, g);
+  const bool active = t >= 0;
   uint32_t nn[L], a[L];
   load_slice_global<L>(nn, M, r);
   if (!CRT) {
@@ -179,12 +151,12 @@ __global__ void __launch_bounds__(NT, MINB) k_modexp(const KeyDev *__restrict__ 
 #pragma unroll
       for (int j = 0; j < L; j++) a[j] = 0;
     }
-    mont<S, TPI, FORM>(a, sR2, nn, n0, r);  // x R mod N
+    mont<S, TPI>(a, sR2, nn, n0, r);  // x R mod N
   } else {
-    crt_input<S, TPI, FORM>(a, in + t * W, active, parts, sR2, sR3, nn, n0, r);
+    crt_input<S, TPI>(a, in + t * W, active, parts, sR2, sR3, nn, n0, r);
   }
-  exp_window<S, TPI, FORM>(a, tbl, ybuf, sched, nsteps, maxidx, nn, n0, r);
-  mont<S, TPI, FORM>(a, sOne, nn, n0, r);  // leave the Montgomery domain
+  exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, nn, n0, r);
+  mont<S, TPI>(a, sOne, nn, n0, r);  // leave the Montgomery domain
   if (active) {
     uint32_t *o = out + t * W + (CRT ? prime * S : 0) + r * L;
     if constexpr (L % 4 == 0) {

@@ -18,7 +18,7 @@ static __device__ __align__(16) uint32_t g_one_row[256] = {1u};
 // memory (the key blob, L1-cached) instead of shared memory; a block then
 // needs only its instances' tables, as many blocks fit per SM as for
 // k_modexp.
-template <int S, int TPI, bool CRT, int FORM, int TABLE = kTableFull>
+template <int S, int TPI, bool CRT, int TABLE = kTableFull>
 __global__ void __launch_bounds__(kThreads) k_modexp_tasks(const BatchTask *__restrict__ tasks, int ntasks,
                                                            int *__restrict__ counter) {
   constexpr int L = S / TPI;
@@ -64,12 +64,12 @@ __global__ void __launch_bounds__(kThreads) k_modexp_tasks(const BatchTask *__re
 #pragma unroll
         for (int j = 0; j < L; j++) a[j] = 0;
       }
-      mont<S, TPI, FORM>(a, sR2, nn, n0, r);
+      mont<S, TPI>(a, sR2, nn, n0, r);
     } else {
-      crt_input<S, TPI, FORM>(a, tk.in + t * W, active, parts, sR2, sR3, nn, n0, r);
+      crt_input<S, TPI>(a, tk.in + t * W, active, parts, sR2, sR3, nn, n0, r);
     }
-    exp_window<S, TPI, FORM>(a, tbl, ybuf, sched, nsteps, maxidx, nn, n0, r);
-    mont<S, TPI, FORM>(a, sOne, nn, n0, r);
+    exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, nn, n0, r);
+    mont<S, TPI>(a, sOne, nn, n0, r);
     if (o) {
       if constexpr (L % 4 == 0) {
 #pragma unroll
@@ -113,8 +113,8 @@ __global__ void __launch_bounds__(kThreads) k_mulmod(const KeyDev *__restrict__ 
   }
   store_slice<L>(yrow, b, r);
   __syncthreads();
-  mont<S, TPI, kChain>(a, yrow, nn, kd.n0, r);
-  mont<S, TPI, kChain>(a, sR2, nn, kd.n0, r);
+  mont<S, TPI>(a, yrow, nn, kd.n0, r);
+  mont<S, TPI>(a, sR2, nn, kd.n0, r);
   if (active) {
     uint32_t *o = out + t * S + r * L;
 #pragma unroll
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kThreads) k_crt_sum(const KeyDev *__restrict__
       for (int o = 1; o < TPI; o <<= 1) any |= __shfl_xor_sync(kFull, any, o, TPI);
     }
     zero = zero || any == 0;
-    mont<S, TPI, kChain>(a, smem + i * ROW, nn, kd.n0, r);  // m_i c_i mod N
+    mont<S, TPI>(a, smem + i * ROW, nn, kd.n0, r);  // m_i c_i mod N
     mod_add<L, TPI>(acc, a, nn, r);
   }
   if (active) {
@@ -190,16 +190,15 @@ constexpr size_t modexp_smem_bytes(int tpi, int threads = kThreads, int table = 
 }  // namespace dev
 
 // One compiled instantiation: limb count, lanes per instance, CRT or full
-// width, Montgomery form (dev::kChain / dev::kCols), odd-power table size
-// (kTableFull / kTableSmall); the one-launch-per-call kernel (round robin,
-// and its twin over key groups) and the persistent batch kernel with their
-// shared-memory sizes.
+// width, odd-power table size (kTableFull / kTableSmall); the
+// one-launch-per-call kernel and the persistent batch kernel with their
+// shared-memory sizes.  forms: the values of pmk_set_kernel_config's form
+// that name it (bit f: form f); every one runs the same kernel.
 struct ModexpEntry {
   int limbs, tpi;
   bool crt;
-  int form;
+  uint32_t forms;
   const void *fn;
-  const void *fn_grp;  // fn over a key group table (same shared memory)
   size_t smem;
   const void *fn_tasks;
   size_t smem_tasks;
@@ -207,29 +206,24 @@ struct ModexpEntry {
   int table;
 };
 
+enum : uint32_t { kForm0 = 1u, kForm01 = 3u };
+
 // NT: block size of the one-launch-per-call kernel.  64 for 32 limbs at 4
 // lanes: a 128-thread block (32 instance tables, 78 KB) leaves two per SM
 // and much shared memory unused, 64-thread blocks fit five (64 -> 80
 // instances per SM): 3.4% faster CRT decryption at 2048 bits and 100 MiB.
 // Other geometries measured no gain or a loss (64 limbs at 4 lanes: 12%
 // slower at 1 MiB) and keep 128.
-// RR_GRP: round-robin launches also take the key-group instantiation (the
-// geometries where it measured faster; see k_modexp).  GRP_MINB: the
-// key-group instantiation's minimum resident blocks per SM, where it differs
-// from MINB (the geometries where it measured faster that way).
-template <int S, int TPI, bool CRT, int FORM, int NT = dev::kThreads, int TABLE = kTableFull, int MINB = 0,
-          bool RR_GRP = false, int GRP_MINB = MINB>
-ModexpEntry make_entry() {
+template <int S, int TPI, bool CRT, int NT = dev::kThreads, int TABLE = kTableFull>
+ModexpEntry make_entry(uint32_t forms) {
   constexpr size_t warp_area = (size_t)(32 / TPI) * dev::Layout<S>::inst(dev::table_rows(TABLE));
   return ModexpEntry{S,
                      TPI,
                      CRT,
-                     FORM,
-                     reinterpret_cast<const void *>(
-                         &dev::k_modexp<S, TPI, CRT, FORM, NT, TABLE, RR_GRP ? GRP_MINB : MINB, RR_GRP>),
-                     reinterpret_cast<const void *>(&dev::k_modexp<S, TPI, CRT, FORM, NT, TABLE, GRP_MINB, true>),
+                     forms,
+                     reinterpret_cast<const void *>(&dev::k_modexp<S, TPI, CRT, NT, TABLE>),
                      dev::modexp_smem_bytes<S>(TPI, NT, TABLE),
-                     reinterpret_cast<const void *>(&dev::k_modexp_tasks<S, TPI, CRT, FORM, TABLE>),
+                     reinterpret_cast<const void *>(&dev::k_modexp_tasks<S, TPI, CRT, TABLE>),
                      sizeof(uint32_t) * warp_area * (dev::kThreads / 32),
                      NT,
                      TABLE};

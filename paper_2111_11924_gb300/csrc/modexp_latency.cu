@@ -7,16 +7,16 @@
 
 namespace pmk {
 
-using dev::kChain;
-using dev::kCols;
-
 const ModexpEntry *modexp_entries_latency(int *count) {
   static const ModexpEntry entries[] = {
-      make_entry<16, 4, true, kChain>(),    make_entry<16, 8, true, kChain>(),
-      make_entry<32, 16, true, kChain>(),   make_entry<32, 16, true, kCols>(),
-      make_entry<64, 32, true, kChain>(),   make_entry<128, 32, true, kChain>(),
-      make_entry<16, 4, false, kChain>(),   make_entry<16, 8, false, kChain>(),
-      make_entry<32, 16, false, kChain>(),  make_entry<32, 16, false, kCols>(),
+      make_entry<16, 4, true>(kForm0),
+      make_entry<16, 8, true>(kForm0),
+      make_entry<32, 16, true>(kForm01),
+      make_entry<64, 32, true>(kForm0),
+      make_entry<128, 32, true>(kForm0),
+      make_entry<16, 4, false>(kForm0),
+      make_entry<16, 8, false>(kForm0),
+      make_entry<32, 16, false>(kForm01),
   };
   *count = (int)(sizeof(entries) / sizeof(entries[0]));
   return entries;

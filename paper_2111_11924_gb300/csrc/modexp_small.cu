@@ -9,25 +9,17 @@
 
 namespace pmk {
 
-using dev::kChain;
-using dev::kCols;
-
 const ModexpEntry *modexp_entries_small(int *count) {
   static const ModexpEntry entries[] = {
-      make_entry<2, 2, true, kChain, dev::kThreads, kTableSmall>(),
-      make_entry<4, 2, true, kChain, dev::kThreads, kTableSmall>(),
-      make_entry<8, 2, true, kChain, dev::kThreads, kTableSmall>(),
-      make_entry<16, 2, true, kChain, dev::kThreads, kTableSmall>(),
-      make_entry<32, 4, true, kChain, 64, kTableSmall>(),
-      make_entry<32, 8, true, kChain, dev::kThreads, kTableSmall>(),
-      make_entry<32, 4, true, kCols, 64, kTableSmall>(),
-      make_entry<32, 8, true, kCols, dev::kThreads, kTableSmall>(),
-      make_entry<48, 8, true, kChain, dev::kThreads, kTableSmall>(),
-      make_entry<48, 8, true, kCols, dev::kThreads, kTableSmall>(),
-      make_entry<64, 8, true, kChain, dev::kThreads, kTableSmall>(),
-      make_entry<64, 16, true, kChain, dev::kThreads, kTableSmall>(),
-      make_entry<64, 8, true, kCols, dev::kThreads, kTableSmall>(),
-      make_entry<64, 16, true, kCols, dev::kThreads, kTableSmall>(),
+      make_entry<2, 2, true, dev::kThreads, kTableSmall>(kForm0),
+      make_entry<4, 2, true, dev::kThreads, kTableSmall>(kForm0),
+      make_entry<8, 2, true, dev::kThreads, kTableSmall>(kForm0),
+      make_entry<16, 2, true, dev::kThreads, kTableSmall>(kForm0),
+      make_entry<32, 4, true, 64, kTableSmall>(kForm01),
+      make_entry<32, 8, true, dev::kThreads, kTableSmall>(kForm01),
+      make_entry<48, 8, true, dev::kThreads, kTableSmall>(kForm01),
+      make_entry<64, 8, true, dev::kThreads, kTableSmall>(kForm01),
+      make_entry<64, 16, true, dev::kThreads, kTableSmall>(kForm01),
   };
   *count = (int)(sizeof(entries) / sizeof(entries[0]));
   return entries;

@@ -5,24 +5,19 @@
 
 namespace pmk {
 
-using dev::kChain;
-using dev::kCols;
-
-// The 192-limb, 16-lane chain geometry (the 6144-bit default) serves its
-// round-robin launches with the key-group instantiation, measured 7% faster
-// at 100 KB and 2.8% at 4 MiB.
 const ModexpEntry *modexp_entries_wide(int *count) {
   static const ModexpEntry entries[] = {
-      make_entry<192, 16, false, kChain, dev::kThreads, kTableFull, 0, true>(),
-      make_entry<192, 16, false, kCols>(),
-      make_entry<256, 16, false, kChain>(), make_entry<256, 16, false, kCols>(),
-      make_entry<256, 32, false, kChain>(), make_entry<96, 8, true, kChain>(),
-      make_entry<96, 16, true, kChain>(),   make_entry<96, 16, true, kCols>(),
-      make_entry<128, 16, true, kChain>(),  make_entry<128, 16, true, kCols>(),
-      // more lanes per instance: shorter exponentiation latency for small batches
-      make_entry<96, 16, false, kChain>(),  make_entry<96, 16, false, kCols>(),
-      make_entry<48, 16, true, kChain>(),   make_entry<128, 32, false, kChain>(),
-      make_entry<192, 32, false, kChain>(), make_entry<64, 32, false, kChain>(),
+      make_entry<192, 16, false>(kForm01),
+      make_entry<256, 16, false>(kForm01),
+      make_entry<256, 32, false>(kForm0),
+      make_entry<96, 8, true>(kForm0),
+      make_entry<96, 16, true>(kForm01),
+      make_entry<128, 16, true>(kForm01),
+      make_entry<96, 16, false>(kForm01),
+      make_entry<48, 16, true>(kForm0),
+      make_entry<128, 32, false>(kForm0),
+      make_entry<192, 32, false>(kForm0),
+      make_entry<64, 32, false>(kForm0),
   };
   *count = (int)(sizeof(entries) / sizeof(entries[0]));
   return entries;

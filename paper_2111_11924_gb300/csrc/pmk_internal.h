@@ -181,9 +181,9 @@ size_t key_groups_words(size_t n, uint32_t K);
 int launch_key_groups(const uint32_t *key_idx, size_t n, uint32_t K, uint32_t align, uint32_t *table,
                       uint32_t *status, cudaStream_t st);
 
-// Launch geometry of an exponentiation kernel: lanes per instance, Montgomery
-// form (0 = one carry chain per lane, 1 = independent columns) and the
-// odd-power table size (kTableFull or kTableSmall; a geometry compiled only
+// Launch geometry of an exponentiation kernel: lanes per instance, form (a
+// name only: forms 0 and 1 of a geometry are one kernel) and the odd-power
+// table size (kTableFull or kTableSmall; a geometry compiled only
 // with the full table runs with it).
 struct KernelConfig {
   uint32_t tpi = 0, form = 0;

@@ -1,6 +1,5 @@
 // Autotuner: for one key set and batch size, time every compiled kernel
-// geometry (lanes per instance x Montgomery form) of the exponentiation that
-// the caller will run, with the full odd-power table (window bound 5) and,
+// geometry (lanes per instance) of the exponentiation that the caller will run, with the full odd-power table (window bound 5) and,
 // where compiled, the small one (bound 4), and keep the fastest in the
 // context.  The window
 // width within the bound is chosen per exponent on the host (fewest
@@ -32,6 +31,7 @@ extern "C" int pmk_autotune(pmk_ctx *ctx, const pmk_keyset *ks, size_t n_chunks,
   for (int table : {pmk::kTableFull, pmk::kTableSmall})
     for (int c = 0; c < ngeom; c++) {
       pmk::KernelConfig k = geoms[c];
+      if (k.form != 0) continue;  // form 1 names the same kernel as form 0
       k.table = table;
       if (table == pmk::kTableFull || pmk::modexp_small_table_built(limbs, k, crt)) cfgs.push_back(k);
     }
