@@ -25,7 +25,7 @@ static_assert(kTableMax >= 16, "the joint tables use rows 0-7 (A) and 8-15 (B)")
 template <int S, int TPI>
 __device__ __forceinline__ void exp2_window(uint32_t (&a)[S / TPI], uint32_t *tbl, uint32_t *ybuf,
                                             const uint32_t *__restrict__ sched, uint32_t nsteps, uint32_t maxa,
-                                            uint32_t maxb, const uint32_t (&nn)[S / TPI], uint32_t n0, uint32_t r) {
+                                            uint32_t maxb, const Modulus<S / TPI> &m, uint32_t r) {
   constexpr int L = S / TPI;
   constexpr int ROW = Layout<S>::kRow;
 #pragma unroll 1
@@ -36,41 +36,54 @@ __device__ __forceinline__ void exp2_window(uint32_t (&a)[S / TPI], uint32_t *tb
     load_slice<L>(a, base, r);
     __syncwarp();
     store_slice<L>(ybuf, a, r);
-    __syncwarp();
-    mont<S, TPI>(a, ybuf, nn, n0, r);  // X^2
-    __syncwarp();
-    store_slice<L>(ybuf, a, r);
-    load_slice<L>(a, base, r);
-    __syncwarp();
+    // k = 0: X^2; k > 0: row k = X^(2k+1)
 #pragma unroll 1
-    for (uint32_t k = 1; k <= maxi; k++) {  // row k = X^(2k+1)
-      mont<S, TPI>(a, ybuf, nn, n0, r);
-      store_slice<L>(base + k * ROW, a, r);
+    for (uint32_t k = 0; k <= maxi; k++) {
+      __syncwarp();
+      mont<S, TPI>(a, ybuf, m, r);
+      if (k == 0) {
+        __syncwarp();
+        store_slice<L>(ybuf, a, r);
+        load_slice<L>(a, base, r);
+      } else {
+        store_slice<L>(base + k * ROW, a, r);
+      }
     }
     __syncwarp();
   }
   __syncwarp();  // rows 0 and 8, stored by the caller, are read whole below
   const uint32_t s0 = __ldg(sched);
-  const uint32_t ia0 = (s0 >> 8) & 0xffu, ib0 = s0 & 0xffu;
-  if (ia0 != 0xffu) {
-    load_slice<L>(a, tbl + ia0 * ROW, r);
-    if (ib0 != 0xffu) mont<S, TPI>(a, tbl + (8 + ib0) * ROW, nn, n0, r);
+  uint32_t si = 0, nsq = 0, ia = (s0 >> 8) & 0xffu, ib = s0 & 0xffu;  // left of step si
+  if (ia != 0xffu) {
+    load_slice<L>(a, tbl + ia * ROW, r);
+    ia = 0xffu;
   } else {
-    load_slice<L>(a, tbl + (8 + ib0) * ROW, r);
+    load_slice<L>(a, tbl + (8 + ib) * ROW, r);
+    ib = 0xffu;
   }
-#pragma unroll 1
-  for (uint32_t si = 1; si < nsteps; si++) {
-    const uint32_t step = __ldg(sched + si);
-    const uint32_t nsq = step >> 16, ia = (step >> 8) & 0xffu, ib = step & 0xffu;
-#pragma unroll 1
-    for (uint32_t k = 0; k < nsq; k++) {
+  for (;;) {  // one product in the code, as in exp_window
+    const uint32_t *y;
+    if (nsq > 0) {
+      nsq--;
       __syncwarp();
       store_slice<L>(ybuf, a, r);
       __syncwarp();
-      mont<S, TPI>(a, ybuf, nn, n0, r);
+      y = ybuf;
+    } else if (ia != 0xffu) {
+      y = tbl + ia * ROW;
+      ia = 0xffu;
+    } else if (ib != 0xffu) {
+      y = tbl + (8 + ib) * ROW;
+      ib = 0xffu;
+    } else {
+      if (++si >= nsteps) break;
+      const uint32_t step = __ldg(sched + si);
+      nsq = step >> 16;
+      ia = (step >> 8) & 0xffu;
+      ib = step & 0xffu;
+      continue;
     }
-    if (ia != 0xffu) mont<S, TPI>(a, tbl + ia * ROW, nn, n0, r);
-    if (ib != 0xffu) mont<S, TPI>(a, tbl + (8 + ib) * ROW, nn, n0, r);
+    mont<S, TPI, true>(a, y, m, r);
   }
 }
 
@@ -79,7 +92,7 @@ __device__ __forceinline__ void exp2_window(uint32_t (&a)[S / TPI], uint32_t *tb
 // parts + i).  With `status`, a c_r divisible by r_i (no inverse mod N)
 // sets kStatusNotInvertible.
 template <int S, int TPI, int NT>
-__global__ void __launch_bounds__(NT) k_blind_crt(const KeyDev *__restrict__ keys, uint32_t K,
+__global__ void __launch_bounds__(NT, 1) k_blind_crt(const KeyDev *__restrict__ keys, uint32_t K,
                                                   const uint32_t *__restrict__ cstar, const uint32_t *__restrict__ cr,
                                                   uint32_t *__restrict__ out, long long n, int parts,
                                                   uint32_t *__restrict__ status) {
@@ -111,12 +124,12 @@ __global__ void __launch_bounds__(NT) k_blind_crt(const KeyDev *__restrict__ key
 
   const long long t = first + (long long)g * K;
   const bool active = t < n;
-  const uint32_t n0 = kd.n0h[prime];
-  uint32_t nn[L], a[L];
-  load_slice_global<L>(nn, kd.P[prime], r);
-  crt_input<S, TPI>(a, cstar + t * W, active, parts, sR2, sR3, nn, n0, r);  // A = c* R mod r_i
+  uint32_t a[L];
+  Modulus<L> m;
+  make_modulus<S, TPI>(m, kd.P[prime], kd.n0h[prime], r);
+  crt_input<S, TPI>(a, cstar + t * W, active, parts, sR2, sR3, m, r);  // A = c* R mod r_i
   store_slice<L>(tbl, a, r);
-  crt_input<S, TPI>(a, cr + t * W, active, parts, sR2, sR3, nn, n0, r);     // B = c_r R mod r_i
+  crt_input<S, TPI>(a, cr + t * W, active, parts, sR2, sR3, m, r);     // B = c_r R mod r_i
   uint32_t any = 0;
 #pragma unroll
   for (int j = 0; j < L; j++) any |= a[j];
@@ -127,8 +140,8 @@ __global__ void __launch_bounds__(NT) k_blind_crt(const KeyDev *__restrict__ key
   if (status && active && r == 0 && any == 0) report(status, kStatusNotInvertible, t);
   store_slice<L>(tbl + 8 * ROW, a, r);
   exp2_window<S, TPI>(a, tbl, ybuf, kd.sched_blind[prime], kd.nsteps_blind[prime], kd.maxa_blind[prime],
-                            kd.maxb_blind[prime], nn, n0, r);
-  mont<S, TPI>(a, sOne, nn, n0, r);  // leave the Montgomery domain
+                            kd.maxb_blind[prime], m, r);
+  mont<S, TPI>(a, sOne, m, r);  // leave the Montgomery domain
   if (active) {
     uint32_t *o = out + t * W + prime * S + r * L;
 #pragma unroll

@@ -24,6 +24,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 
 #include "pmk_internal.h"
 
@@ -109,11 +110,10 @@ __device__ __forceinline__ uint32_t lookahead(bool gen, bool prop, bool top) {
   return (cin >> (threadIdx.x & 31)) & 1u;
 }
 
-// Resolve the pending word c0 (lane r's belongs at lane r+1's limb 0; the top
-// lane's is the value's top word) and reduce the value once by N, leaving the
-// canonical result (< N) in t.  Requires the value < 2N.
+// Resolve the pending word c0 of every lane (lane r's belongs at lane r+1's
+// limb 0) into t.  Returns the value's word above limb S - 1 (top lane only).
 template <int L, int TPI>
-__device__ __forceinline__ void finalize(uint32_t (&t)[L], uint32_t c0, const uint32_t (&nn)[L], uint32_t r) {
+__device__ __forceinline__ uint32_t resolve(uint32_t (&t)[L], uint32_t c0, uint32_t r) {
   const bool top = (r == TPI - 1);
   uint32_t topw = top ? c0 : 0u;
   if constexpr (TPI > 1) {
@@ -135,6 +135,14 @@ __device__ __forceinline__ void finalize(uint32_t (&t)[L], uint32_t c0, const ui
     addc(g2, 0u, 0u);
     if (top) topw += g + g2;
   }
+  return topw;
+}
+
+// Subtract N once if the value (topw above t, topw in the top lane) is at
+// least N.  Returns the new word above limb S - 1 (top lane only).
+template <int L, int TPI>
+__device__ __forceinline__ uint32_t reduce_once(uint32_t (&t)[L], uint32_t topw, const uint32_t (&nn)[L], uint32_t r) {
+  const bool top = (r == TPI - 1);
   uint32_t d[L], b;
   sub_cc(d[0], t[0], nn[0]);
 #pragma unroll
@@ -159,233 +167,17 @@ __device__ __forceinline__ void finalize(uint32_t (&t)[L], uint32_t c0, const ui
   if (ge) {
 #pragma unroll
     for (int j = 0; j < L; j++) t[j] = d[j];
+    topw -= b;
   }
+  return topw;
 }
 
-// Rows of a product per unrolled group.  A group of L rows (or 2 L, for whole
-// 16-byte reads of y) brings the per-row shift of the lane's words back to
-// the starting registers, so no register moves remain.
-template <int S, int L>
-__host__ __device__ constexpr int row_group() {
-  return (L % 4 == 0) ? L : (L % 2 == 0 && S % (2 * L) == 0) ? 2 * L : (L % 2 == 0) ? L : (S % 4 == 0) ? 4 : 2;
-}
-
-template <int K>
-__device__ __forceinline__ void load_y(uint32_t (&yv)[K], const uint32_t *ys) {
-  if constexpr (K % 4 == 0) {
-#pragma unroll
-    for (int q = 0; q < K; q += 4) {
-      const uint4 v = *reinterpret_cast<const uint4 *>(ys + q);
-      yv[q] = v.x; yv[q + 1] = v.y; yv[q + 2] = v.z; yv[q + 3] = v.w;
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < K; q += 2) {
-      const uint2 v = *reinterpret_cast<const uint2 *>(ys + q);
-      yv[q] = v.x; yv[q + 1] = v.y;
-    }
-  }
-}
-
-// a <- MontMul(a, y) = a y R^-1 mod N.  a: this lane's limbs (any value < R);
-// ys: y's S limbs in shared memory (y < N), read as 16-byte broadcasts.
-// One row at a time, one add-with-carry chain per lane: the form for an odd
-// number of limbs per lane, which has no pairs.
-template <int S, int TPI>
-__device__ __forceinline__ void mont_mul(uint32_t (&a)[S / TPI], const uint32_t *ys, const uint32_t (&nn)[S / TPI],
-                                         uint32_t n0, uint32_t r) {
-  constexpr int L = S / TPI;
-  constexpr int kStep = row_group<S, L>();
-  uint32_t t[L];
-#pragma unroll
-  for (int j = 0; j < L; j++) t[j] = 0;
-  uint32_t c0 = 0, c1 = 0;
-#pragma unroll 1
-  for (int i0 = 0; i0 < S; i0 += kStep) {
-    uint32_t yv[kStep];
-    load_y<kStep>(yv, ys + i0);
-#pragma unroll
-    for (int u = 0; u < kStep; u++) {
-      row_mac<L>(t, c0, c1, a, yv[u]);
-      uint32_t q = t[0] * n0;
-      if constexpr (TPI > 1) q = __shfl_sync(kFull, q, 0, TPI);
-      row_mac<L>(t, c0, c1, nn, q);
-      // T /= 2^32: limb 0 of lane 0 is now zero; every lane takes the next
-      // lane's limb 0 as its new top limb and folds its pending word into it.
-      uint32_t in = 0;
-      if constexpr (TPI > 1) {
-        in = __shfl_down_sync(kFull, t[0], 1, TPI);
-        if (r == TPI - 1) in = 0;
-      }
-#pragma unroll
-      for (int j = 0; j < L - 1; j++) t[j] = t[j + 1];
-      add_cc(t[L - 1], in, c0);
-      addc(c0, c1, 0u);
-      c1 = 0;
-    }
-  }
-  finalize<L, TPI>(t, c0, nn, r);
-#pragma unroll
-  for (int j = 0; j < L; j++) a[j] = t[j];
-}
-
-// (lo, hi) += a y, a 64-bit pair, with the carry out (and in, for madc) in the
-// condition code; each compiles to one wide multiply-add.
-__device__ __forceinline__ void mad_wide_cc(uint32_t &lo, uint32_t &hi, uint32_t a, uint32_t y) {
-  asm volatile("mad.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.cc.u32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(y));
-}
-__device__ __forceinline__ void madc_wide_cc(uint32_t &lo, uint32_t &hi, uint32_t a, uint32_t y) {
-  asm volatile("madc.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.cc.u32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(y));
-}
-
-// (w[OFF + 2 i], w[OFF + 2 i + 1]) += m[PAR + 2 i] y for i < L / 2 in one
-// carry chain.  CIN: the chain takes the condition code's carry.  The carry
-// out is left in the condition code.
-template <int L, int PAR, int OFF, bool CIN, int W>
-__device__ __forceinline__ void pair_chain(uint32_t (&w)[W], const uint32_t (&m)[L], uint32_t y) {
-  if constexpr (CIN) {
-    madc_wide_cc(w[OFF], w[OFF + 1], m[PAR], y);
-  } else {
-    mad_wide_cc(w[OFF], w[OFF + 1], m[PAR], y);
-  }
-#pragma unroll
-  for (int i = 1; i < L / 2; i++) madc_wide_cc(w[OFF + 2 * i], w[OFF + 2 * i + 1], m[PAR + 2 * i], y);
-}
-
-// a <- MontMul(a, y) for an even number of limbs per lane: two rows per step.
-//
-// The lane's part of T is kept as two sums of 64-bit pairs: e, whose word j
-// has weight 2^(32 j), and o, whose word j has weight 2^(32 (j + 1)).  The
-// even limbs times y_i and the odd limbs times y_{i+1} land on e's pairs, the
-// other two products on o's, so each of the four is one carry chain of L / 2
-// wide multiply-adds.  The quotient of both rows is one 64-bit value,
-// q = T (-N^-1) mod 2^64 of lane 0, and T /= 2^64 moves whole pairs: e and o
-// keep their roles and a step needs one broadcast of q and one shift between
-// lanes.  A chain's carry out is held back (c0, c1, c2: weights L, L + 1,
-// L + 2) and joins the words that the shift brings in.
-//
-// Bound: the wide multiply-add, 4 L per lane and step against about 26 other
-// instructions on other pipes.  Measured against the column form that it
-// replaces (2048-bit keys, full d): 12.76 vs 17.67 ms at 1 MiB, 104.9 vs
-// 142.7 ms at 10 MiB; CRT 3.41 vs 4.64 ms at 1 MiB.
-template <int S, int TPI>
-__device__ __forceinline__ void mont_mul_pairs(uint32_t (&a)[S / TPI], const uint32_t *ys,
-                                               const uint32_t (&nn)[S / TPI], uint32_t n0, uint32_t r) {
-  constexpr int L = S / TPI;
-  static_assert(L % 2 == 0, "pairs of limbs");
-  constexpr int kStep = row_group<S, L>();
-  // -N^-1 mod 2^64 from its low word by one Newton step (lane 0's is used).
-  const uint64_t n01 = ((uint64_t)nn[1] << 32) | nn[0];
-  const uint32_t k1 = (uint32_t)(((uint64_t)n0 * (2 + n01 * n0)) >> 32);
-  const uint32_t below_top = (r == TPI - 1) ? 0u : kFull;
-  uint32_t e[L + 2], o[L];
-#pragma unroll
-  for (int j = 0; j < L; j++) e[j] = o[j] = 0;
-  e[L] = e[L + 1] = 0;
-  uint32_t c0 = 0, c1 = 0, c2 = 0;
-  // The words of weight 0 and 1 go to the lane below (lane 0's are zero).
-  auto shifted_out = [&](uint32_t &x0, uint32_t &x1) {
-    x0 = e[0];
-    x1 = e[1] + o[0];
-    if constexpr (TPI > 1) {
-      x0 = __shfl_down_sync(kFull, x0, 1, TPI) & below_top;
-      x1 = __shfl_down_sync(kFull, x1, 1, TPI) & below_top;
-    } else {
-      x0 = x1 = 0;
-    }
-  };
-#pragma unroll 1
-  for (int i0 = 0; i0 < S; i0 += kStep) {
-    uint32_t yv[kStep];
-    load_y<kStep>(yv, ys + i0);
-#pragma unroll
-    for (int u = 0; u < kStep; u += 2) {
-      // T /= 2^64.  o's first pair ends in weight 2; the carry of that sum has
-      // weight 3, the first word of the new o, where the next chain starts.
-      uint32_t x0, x1, drop;
-      shifted_out(x0, x1);
-      add_cc(drop, e[1], o[0]);
-      addc_cc(e[2], e[2], o[1]);
-      uint32_t f[L + 2], p[L];
-#pragma unroll
-      for (int j = 0; j < L; j++) f[j] = e[j + 2];
-#pragma unroll
-      for (int j = 0; j < L - 2; j++) p[j] = o[j + 2];
-      p[L - 2] = p[L - 1] = 0;
-      pair_chain<L, 1, 0, true>(p, a, yv[u]);
-      uint32_t d1;
-      addc(d1, 0u, 0u);
-      add_cc(f[L - 2], f[L - 2], c0);
-      addc_cc(f[L - 1], f[L - 1], c1);
-      addc(c2, c2, 0u);
-      add_cc(f[L - 2], f[L - 2], x0);
-      addc_cc(f[L - 1], f[L - 1], x1);
-      addc(f[L], c2, 0u);
-      // T += a (y_i + 2^32 y_{i+1})
-      pair_chain<L, 0, 0, false>(f, a, yv[u]);
-      addc(f[L], f[L], 0u);
-      pair_chain<L, 0, 0, false>(p, a, yv[u + 1]);
-      addc(f[L + 1], d1, 0u);
-      uint32_t q0 = f[0] * n0;
-      uint32_t q1 = __umulhi(f[0], n0) + f[0] * k1 + (f[1] + p[0]) * n0;
-      if constexpr (TPI > 1) {
-        q0 = __shfl_sync(kFull, q0, 0, TPI);
-        q1 = __shfl_sync(kFull, q1, 0, TPI);
-      }
-      pair_chain<L, 1, 2, false>(f, a, yv[u + 1]);
-      addc(c2, 0u, 0u);
-      // T += N (q_0 + 2^32 q_1)
-      pair_chain<L, 0, 0, false>(f, nn, q0);
-      addc(c0, 0u, 0u);
-      pair_chain<L, 1, 0, false>(p, nn, q0);
-      addc(c1, 0u, 0u);
-      pair_chain<L, 0, 0, false>(p, nn, q1);
-      addc(c1, c1, 0u);
-      pair_chain<L, 1, 2, false>(f, nn, q1);
-      addc(c2, c2, 0u);
-#pragma unroll
-      for (int j = 0; j < L + 2; j++) e[j] = f[j];
-#pragma unroll
-      for (int j = 0; j < L; j++) o[j] = p[j];
-    }
-  }
-  // The last shift, then e and o in one carry chain.
-  uint32_t x0, x1, drop;
-  shifted_out(x0, x1);
-  add_cc(e[L], e[L], c0);
-  addc_cc(e[L + 1], e[L + 1], c1);
-  addc(c2, c2, 0u);
-  add_cc(e[L], e[L], x0);
-  addc_cc(e[L + 1], e[L + 1], x1);
-  addc(c2, c2, 0u);
-  add_cc(drop, e[1], o[0]);
-#pragma unroll
-  for (int j = 0; j < L; j++) addc_cc(a[j], e[j + 2], (j + 1 < L) ? o[j + 1] : 0u);
-  addc(c2, c2, 0u);
-  finalize<L, TPI>(a, c2, nn, r);
-}
-
-template <int S, int TPI>
-__device__ __forceinline__ void mont(uint32_t (&a)[S / TPI], const uint32_t *ys, const uint32_t (&nn)[S / TPI],
-                                     uint32_t n0, uint32_t r) {
-  if constexpr ((S / TPI) % 2 == 0) {
-    mont_mul_pairs<S, TPI>(a, ys, nn, n0, r);
-  } else {
-    mont_mul<S, TPI>(a, ys, nn, n0, r);
-  }
-}
-
-// a <- (a + b) mod N for a, b < N (distributed add, lookahead, one reduction).
+// Resolve pending words and reduce the value once by N, leaving the canonical
+// result (< N) in t.  Requires the value < 2N.
 template <int L, int TPI>
-__device__ __forceinline__ void mod_add(uint32_t (&a)[L], const uint32_t (&b)[L], const uint32_t (&nn)[L], uint32_t r) {
-  uint32_t c;
-  add_cc(a[0], a[0], b[0]);
-#pragma unroll
-  for (int j = 1; j < L; j++) addc_cc(a[j], a[j], b[j]);
-  addc(c, 0u, 0u);
-  // c is this lane's carry into the next lane: reuse finalize, whose first
-  // step moves a lane's pending word into the next lane's limb 0.
-  finalize<L, TPI>(a, c, nn, r);
+__device__ __forceinline__ void finalize(uint32_t (&t)[L], uint32_t c0, const uint32_t (&nn)[L], uint32_t r) {
+  const uint32_t topw = resolve<L, TPI>(t, c0, r);
+  reduce_once<L, TPI>(t, topw, nn, r);
 }
 
 // Store / load this lane's L limbs of a value at row + r L.
@@ -429,46 +221,519 @@ __device__ __forceinline__ void load_slice_global(uint32_t (&a)[L], const uint32
   }
 }
 
+// A modulus N as the products use it: this lane's limbs of N, and for two or
+// more limbs per lane (see PairSum) of F = (k N + 1) / 2^64 with
+// k = -N^-1 mod 2^64.  tight: N is so near 2^(32 S) that a product can reach
+// 2N before its last subtraction.
+template <int L>
+struct Modulus {
+  uint32_t n[L], f[L];
+  uint32_t k0, k1;
+  bool tight;
+};
+
+// a <- MontMul(a, y) = a y R^-1 mod N.  a: this lane's limbs (any value < R);
+// ys: y's S limbs in shared memory (y < N), read as 16-byte broadcasts.
+// One row at a time, one add-with-carry chain per lane: the form for one limb
+// per lane (the residues of 128-bit keys), which has no pairs.
+template <int S, int TPI>
+__device__ __forceinline__ void mont_mul_chain(uint32_t (&a)[S / TPI], const uint32_t *ys, const Modulus<S / TPI> &m,
+                                               uint32_t r) {
+  constexpr int L = S / TPI;
+  uint32_t t[L];
+#pragma unroll
+  for (int j = 0; j < L; j++) t[j] = 0;
+  uint32_t c0 = 0, c1 = 0;
+  constexpr int kStep = (S % 4 == 0) ? 4 : 2;  // rows per 16- or 8-byte read of y
+#pragma unroll 1
+  for (int i0 = 0; i0 < S; i0 += kStep) {
+    uint32_t yv[kStep];
+    load_slice<kStep>(yv, ys + i0, 0);
+#pragma unroll
+    for (int u = 0; u < kStep; u++) {
+      row_mac<L>(t, c0, c1, a, yv[u]);
+      uint32_t q = t[0] * m.k0;
+      if constexpr (TPI > 1) q = __shfl_sync(kFull, q, 0, TPI);
+      row_mac<L>(t, c0, c1, m.n, q);
+      // T /= 2^32: limb 0 of lane 0 is now zero; every lane takes the next
+      // lane's limb 0 as its new top limb and folds its pending word into it.
+      uint32_t in = 0;
+      if constexpr (TPI > 1) {
+        in = __shfl_down_sync(kFull, t[0], 1, TPI);
+        if (r == TPI - 1) in = 0;
+      }
+#pragma unroll
+      for (int j = 0; j < L - 1; j++) t[j] = t[j + 1];
+      add_cc(t[L - 1], in, c0);
+      addc(c0, c1, 0u);
+      c1 = 0;
+    }
+  }
+  finalize<L, TPI>(t, c0, m.n, r);
+#pragma unroll
+  for (int j = 0; j < L; j++) a[j] = t[j];
+}
+
+// (lo, hi) += a y, a 64-bit pair, with the carry out (and in, for madc) in the
+// condition code; each compiles to one wide multiply-add.
+__device__ __forceinline__ void mad_wide_cc(uint32_t &lo, uint32_t &hi, uint32_t a, uint32_t y) {
+  asm volatile("mad.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.cc.u32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(y));
+}
+__device__ __forceinline__ void madc_wide_cc(uint32_t &lo, uint32_t &hi, uint32_t a, uint32_t y) {
+  asm volatile("madc.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.cc.u32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(y));
+}
+
+// (w[OFF + 2 i], w[OFF + 2 i + 1]) += m[PAR + 2 i] y over the limbs of one
+// parity (PAR) in one carry chain.  CIN: the chain takes the condition code's
+// carry.  The carry out is left in the condition code.
+template <int L, int PAR, int OFF, bool CIN = false, int W>
+__device__ __forceinline__ void pair_chain(uint32_t (&w)[W], const uint32_t (&m)[L], uint32_t y) {
+  if constexpr (CIN) {
+    madc_wide_cc(w[OFF], w[OFF + 1], m[PAR], y);
+  } else {
+    mad_wide_cc(w[OFF], w[OFF + 1], m[PAR], y);
+  }
+#pragma unroll
+  for (int i = 1; i < (L + 1 - PAR) / 2; i++) madc_wide_cc(w[OFF + 2 * i], w[OFF + 2 * i + 1], m[PAR + 2 * i], y);
+}
+
+// pair_chain whose last pair starts from zero.
+template <int L, int PAR, int W>
+__device__ __forceinline__ void pair_chain_new_top(uint32_t (&w)[W], const uint32_t (&m)[L], uint32_t y) {
+#pragma unroll
+  for (int i = 0; i < L / 2 - 1; i++) madc_wide_cc(w[2 * i], w[2 * i + 1], m[PAR + 2 * i], y);
+  asm volatile("madc.lo.cc.u32 %0, %2, %3, 0;\n\tmadc.hi.cc.u32 %1, %2, %3, 0;"
+               : "=r"(w[L - 2]), "=r"(w[L - 1])
+               : "r"(m[PAR + L - 2]), "r"(y));
+}
+
+__device__ __forceinline__ void mul_wide(uint32_t &lo, uint32_t &hi, uint32_t a, uint32_t y) {
+  const uint64_t p = (uint64_t)a * y;
+  lo = (uint32_t)p;
+  hi = (uint32_t)(p >> 32);
+}
+
+// The running sum T of a Montgomery product for an even number of limbs per
+// lane, two rows (64 bits of y) a step.
+//
+// A lane's part of T is two sums of 64-bit pairs: e, whose word j has weight
+// 2^(32 j), and o, whose word j has weight 2^(32 (j + 1)).  The even limbs
+// times y_i and the odd limbs times y_{i+1} land on e's pairs, the other two
+// products on o's, so each of the four is one carry chain of L / 2 wide
+// multiply-adds, and T / 2^64 moves whole pairs: e and o keep their roles.
+//
+// Reduction.  F = (k N + 1) / 2^64 with k = -N^-1 mod 2^64 makes
+// k N = F 2^64 - 1, so adding T mod 2^64 times k N clears the low 64 bits:
+//     T <- floor(T / 2^64) + (T mod 2^64) F.
+// The quotient is lane 0's two low words as they stand, with no product by k
+// on the way, and F has no more limbs than N.  T stays below
+// (2^64 + 1) N + a; the last two steps therefore reduce by N itself
+// (q = T k mod 2^64), which brings T below 2N, or below 3N when the top 64
+// bits of N are all but ones (Modulus::tight).
+//
+// Chains are ordered so that each one's carry out falls on a word that holds
+// only carries yet.  The two words a lane passes down and the next quotient
+// are sent before a step's last two chains, which hide the shuffles.
+template <int L, int TPI>
+struct PairSum {
+  uint32_t e[L + 2], o[L], c2;  // c2: weight 2^(32 (L + 2))
+  uint32_t x0, x1, q0, q1;      // from the lane above (its words 0, 1), and the quotient
+  uint32_t below_top;           // all ones except in the top lane
+
+  __device__ __forceinline__ explicit PairSum(uint32_t r) : below_top(r == TPI - 1 ? 0u : kFull) {}
+
+  template <bool QUOTIENT>
+  __device__ __forceinline__ void send() {
+    x0 = e[0];
+    x1 = e[1] + o[0];
+    if constexpr (TPI > 1) {
+      if constexpr (QUOTIENT) {
+        q0 = __shfl_sync(kFull, x0, 0, TPI);
+        q1 = __shfl_sync(kFull, x1, 0, TPI);
+      }
+      x0 = __shfl_down_sync(kFull, x0, 1, TPI);
+      x1 = __shfl_down_sync(kFull, x1, 1, TPI);
+    } else {
+      q0 = x0;
+      q1 = x1;
+      x0 = x1 = 0;
+    }
+  }
+
+  // T = a (y0 + 2^32 y1)
+  __device__ __forceinline__ void start(const uint32_t (&a)[L], uint32_t y0, uint32_t y1) {
+#pragma unroll
+    for (int j = 0; j < L; j += 2) {
+      mul_wide(e[j], e[j + 1], a[j], y0);
+      mul_wide(o[j], o[j + 1], a[j + 1], y0);
+    }
+    pair_chain<L, 0, 0>(o, a, y1);
+    addc(e[L + 1], 0u, 0u);
+    e[L] = 0;
+    send<true>();
+    pair_chain<L, 1, 2>(e, a, y1);
+    c2 = 0;
+  }
+
+  // T = T / 2^64 + a (y0 + 2^32 y1), and with REDUCE + (q0 + 2^32 q1) f.
+  template <bool REDUCE>
+  __device__ __forceinline__ void step(const uint32_t (&a)[L], uint32_t y0, uint32_t y1, const uint32_t (&f)[L]) {
+    uint32_t d, drop;  // d: weight L + 1
+    // o's first pair ends in weight 2, the new weight 0; the carry of that
+    // sum has the new weight 1, where o's next chain starts.
+    add_cc(drop, e[1], o[0]);
+    addc_cc(e[2], e[2], o[1]);
+#pragma unroll
+    for (int j = 0; j < L - 2; j++) o[j] = o[j + 2];
+    pair_chain_new_top<L, 1>(o, a, y0);
+    addc(d, 0u, 0u);
+#pragma unroll
+    for (int j = 0; j < L; j++) e[j] = e[j + 2];
+    pair_chain<L, 0, 0>(e, a, y0);
+    addc(e[L], c2, 0u);
+    pair_chain<L, 0, 0>(o, a, y1);
+    addc(d, d, 0u);
+    add_cc(e[L - 2], e[L - 2], x0 & below_top);
+    addc_cc(e[L - 1], e[L - 1], x1 & below_top);
+    addc(e[L], e[L], 0u);
+    if constexpr (REDUCE) {
+      pair_chain<L, 0, 0>(e, f, q0);
+      addc(e[L], e[L], 0u);
+      pair_chain<L, 1, 0>(o, f, q0);
+      addc(d, d, 0u);
+      const uint32_t p1 = q1;
+      pair_chain<L, 0, 0>(o, f, p1);
+      addc(e[L + 1], d, 0u);
+      send<true>();
+      pair_chain<L, 1, 2>(e, a, y1);
+      addc(c2, 0u, 0u);
+      pair_chain<L, 1, 2>(e, f, p1);
+      addc(c2, c2, 0u);
+    } else {
+      e[L + 1] = d;
+      pair_chain<L, 1, 2>(e, a, y1);
+      addc(c2, 0u, 0u);
+    }
+  }
+
+  // T += q N with q = T (-N^-1) mod 2^64
+  __device__ __forceinline__ void reduce(const Modulus<L> &m) {
+    const uint64_t w = (uint64_t)e[0] * m.k0;
+    uint32_t p0 = (uint32_t)w;
+    uint32_t p1 = (uint32_t)(w >> 32) + e[0] * m.k1 + (e[1] + o[0]) * m.k0;
+    if constexpr (TPI > 1) {
+      p0 = __shfl_sync(kFull, p0, 0, TPI);
+      p1 = __shfl_sync(kFull, p1, 0, TPI);
+    }
+    uint32_t c0, c1;  // carries of weight L and L + 1, whose words are full here
+    pair_chain<L, 0, 0>(e, m.n, p0);
+    addc(c0, 0u, 0u);
+    pair_chain<L, 1, 0>(o, m.n, p0);
+    addc(c1, 0u, 0u);
+    pair_chain<L, 0, 0>(o, m.n, p1);
+    addc(c1, c1, 0u);
+    send<false>();
+    pair_chain<L, 1, 2>(e, m.n, p1);
+    addc(c2, c2, 0u);
+    add_cc(e[L], e[L], c0);
+    addc_cc(e[L + 1], e[L + 1], c1);
+    addc(c2, c2, 0u);
+  }
+
+  // t = T / 2^64 (rounded down); returns the lane's pending word.
+  __device__ __forceinline__ uint32_t shift_out(uint32_t (&t)[L]) {
+    uint32_t drop, c;
+    add_cc(e[L], e[L], x0 & below_top);
+    addc_cc(e[L + 1], e[L + 1], x1 & below_top);
+    addc(c, c2, 0u);
+    add_cc(drop, e[1], o[0]);
+#pragma unroll
+    for (int j = 0; j < L; j++) addc_cc(t[j], e[j + 2], (j + 1 < L) ? o[j + 1] : 0u);
+    addc(c, c, 0u);
+    return c;
+  }
+};
+
+// PairSum for an odd number of limbs per lane (3 or more).  The even limbs are
+// one more than the odd ones, so e ends in weight L and o in weight L + 1, and
+// the words that hold only carries are others: the chains' order differs.
+template <int L, int TPI>
+struct OddPairSum {
+  uint32_t e[L + 1], o[L + 1], c1, c2;  // c1, c2: weights 2^(32 (L + 1)), 2^(32 (L + 2))
+  uint32_t x0, x1, q0, q1;
+  uint32_t below_top;
+
+  __device__ __forceinline__ explicit OddPairSum(uint32_t r) : below_top(r == TPI - 1 ? 0u : kFull) {}
+
+  template <bool QUOTIENT>
+  __device__ __forceinline__ void send() {
+    x0 = e[0];
+    x1 = e[1] + o[0];
+    if constexpr (QUOTIENT) {
+      q0 = __shfl_sync(kFull, x0, 0, TPI);
+      q1 = __shfl_sync(kFull, x1, 0, TPI);
+    }
+    x0 = __shfl_down_sync(kFull, x0, 1, TPI);
+    x1 = __shfl_down_sync(kFull, x1, 1, TPI);
+  }
+
+  __device__ __forceinline__ void start(const uint32_t (&a)[L], uint32_t y0, uint32_t y1) {
+#pragma unroll
+    for (int j = 0; j < L; j += 2) mul_wide(e[j], e[j + 1], a[j], y0);
+#pragma unroll
+    for (int j = 1; j < L; j += 2) mul_wide(o[j - 1], o[j], a[j], y0);
+    o[L - 1] = o[L] = 0;
+    pair_chain<L, 0, 0>(o, a, y1);
+    c2 = 0;  // a (y0 + 2^32 y1) ends below weight L + 2
+    send<true>();
+    pair_chain<L, 1, 2>(e, a, y1);
+    addc(c1, 0u, 0u);
+  }
+
+  template <bool REDUCE>
+  __device__ __forceinline__ void step(const uint32_t (&a)[L], uint32_t y0, uint32_t y1, const uint32_t (&f)[L]) {
+    uint32_t drop, d;  // d: weight L + 1
+    add_cc(drop, e[1], o[0]);
+    addc_cc(e[2], e[2], o[1]);
+#pragma unroll
+    for (int j = 0; j < L - 1; j++) o[j] = o[j + 2];
+    pair_chain<L, 1, 0, true>(o, a, y0);
+    addc(o[L - 1], 0u, 0u);
+#pragma unroll
+    for (int j = 0; j < L - 1; j++) e[j] = e[j + 2];
+    e[L - 1] = c1;
+    e[L] = c2;
+    pair_chain<L, 0, 0>(e, a, y0);
+    addc(d, 0u, 0u);
+    add_cc(e[L - 2], e[L - 2], x0 & below_top);
+    addc_cc(e[L - 1], e[L - 1], x1 & below_top);
+    addc_cc(e[L], e[L], 0u);
+    addc(d, d, 0u);
+    if constexpr (REDUCE) {
+      pair_chain<L, 0, 0>(e, f, q0);
+      addc(d, d, 0u);
+      pair_chain<L, 1, 0>(o, f, q0);
+      addc(o[L - 1], o[L - 1], 0u);
+    }
+    o[L] = d;
+    pair_chain<L, 0, 0>(o, a, y1);
+    addc(c2, 0u, 0u);
+    if constexpr (REDUCE) {
+      const uint32_t p1 = q1;
+      pair_chain<L, 0, 0>(o, f, p1);
+      addc(c2, c2, 0u);
+      send<true>();
+      pair_chain<L, 1, 2>(e, a, y1);
+      addc(c1, 0u, 0u);
+      pair_chain<L, 1, 2>(e, f, p1);
+      addc(c1, c1, 0u);
+    } else {
+      pair_chain<L, 1, 2>(e, a, y1);
+      addc(c1, 0u, 0u);
+    }
+  }
+
+  __device__ __forceinline__ void reduce(const Modulus<L> &m) {
+    const uint64_t w = (uint64_t)e[0] * m.k0;
+    uint32_t p0 = (uint32_t)w;
+    uint32_t p1 = (uint32_t)(w >> 32) + e[0] * m.k1 + (e[1] + o[0]) * m.k0;
+    p0 = __shfl_sync(kFull, p0, 0, TPI);
+    p1 = __shfl_sync(kFull, p1, 0, TPI);
+    uint32_t c0;  // weight L, whose words are full here
+    pair_chain<L, 0, 0>(e, m.n, p0);
+    addc(c1, c1, 0u);
+    pair_chain<L, 1, 0>(o, m.n, p0);
+    addc(c0, 0u, 0u);
+    pair_chain<L, 0, 0>(o, m.n, p1);
+    addc(c2, c2, 0u);
+    send<false>();
+    pair_chain<L, 1, 2>(e, m.n, p1);
+    addc(c1, c1, 0u);
+    add_cc(o[L - 1], o[L - 1], c0);
+    addc_cc(o[L], o[L], 0u);
+    addc(c2, c2, 0u);
+  }
+
+  __device__ __forceinline__ uint32_t shift_out(uint32_t (&t)[L]) {
+    uint32_t drop, c;
+    add_cc(e[L], e[L], x0 & below_top);
+    addc_cc(o[L], o[L], x1 & below_top);
+    addc(c, c2, 0u);
+    add_cc(o[L], o[L], c1);
+    addc(c, c, 0u);
+    add_cc(drop, e[1], o[0]);
+#pragma unroll
+    for (int j = 0; j < L; j++) addc_cc(t[j], (j + 2 <= L) ? e[j + 2] : 0u, o[j + 1]);
+    addc(c, c, 0u);
+    return c;
+  }
+};
+
+template <int S, int TPI>
+__device__ __forceinline__ void make_modulus(Modulus<S / TPI> &m, const uint32_t *N, uint32_t n0, uint32_t r) {
+  constexpr int L = S / TPI;
+  load_slice_global<L>(m.n, N, r);
+  m.k0 = n0;
+  m.tight = false;
+  if constexpr (L > 1) {
+    // -N^-1 mod 2^64 from its low word by one Newton step, in lane 0
+    const uint64_t n01 = ((uint64_t)m.n[1] << 32) | m.n[0];
+    m.k1 = (uint32_t)(((uint64_t)n0 * (2 + n01 * n0)) >> 32);
+    if constexpr (TPI > 1) m.k1 = __shfl_sync(kFull, m.k1, 0, TPI);
+    std::conditional_t<L % 2 == 0, PairSum<L, TPI>, OddPairSum<L, TPI>> t(r);
+    t.start(m.n, m.k0, m.k1);
+    const uint32_t c = t.shift_out(m.f);
+    // k N = -1 mod 2^64: the + 1 carries out of the dropped words into lane 0
+    uint32_t g;
+    add_cc(m.f[0], m.f[0], r == 0 ? 1u : 0u);
+#pragma unroll
+    for (int j = 1; j < L; j++) addc_cc(m.f[j], m.f[j], 0u);
+    addc(g, c, 0u);
+    resolve<L, TPI>(m.f, g, r);
+    uint32_t t1 = m.n[L - 1], t0 = m.n[L - 2];
+    if constexpr (TPI > 1) {
+      t1 = __shfl_sync(kFull, t1, TPI - 1, TPI);
+      t0 = __shfl_sync(kFull, t0, TPI - 1, TPI);
+    }
+    m.tight = t1 == 0xffffffffu && t0 >= 0xfffffff0u;  // T < 2N needs the top 64 bits of N below 2^64 - 5
+  }
+}
+
+// Steps of a product unrolled together.  HOT is the exponentiation's own
+// product (one site per kernel), unrolled whole where that still measured
+// faster; elsewhere as many steps as bring a lane's words back to the
+// registers they started from.  Clocks per product with 1 / 2 / 3 warps per
+// scheduler, L / 2 steps against the whole product: 64 limbs on 32 lanes
+// 3,316 / 4,765 / 6,913 and 2,504 / 3,763 / 5,197, on 16 lanes 4,581 / 6,572 /
+// 9,568 and 3,835 / 5,684 / 8,433, on 8 lanes 7,279 / 10,376 / 16,009 and
+// 6,860 / 9,863 / 15,620; 32 limbs on 4 lanes 3,917 / 5,511 and 3,711 / 5,245.
+template <int S, int L, bool HOT>
+__host__ __device__ constexpr int unrolled_steps() {
+  return !HOT                                                ? (L == 2 ? 2 : L % 2 ? L : L / 2)
+         : (S <= 96 && L <= 12) || (S == 128 && L <= 4)      ? S / 2 - 2
+         : L % 2 == 0 && 12 % (L / 2) == 0                   ? 12
+                                                             : L / 2;
+}
+
+// a <- MontMul(a, y) = a y R^-1 mod N for two or more limbs per lane.
+// a: any value < R; ys: y's S limbs in shared or global memory (y < N).
+//
+// Bound: the wide multiply-add, 4 L per lane and step at 4 clocks of the
+// fma-heavy pipe each, against about 20 other instructions a step; a single
+// warp issues one per 6.6 clocks, two nearly fill the pipe.  Measured (2048-bit
+// keys, full d, default geometry): 1 MiB
+// 17.63 ms with 64-bit columns, 12.66 with two-row steps and a quotient by
+// product, 11.68 now; 10 MiB 142.3, 104.1, 94.6; CRT 1 MiB 4.63, 3.34, 3.10.
+template <int S, int TPI, bool HOT>
+__device__ __forceinline__ void mont_mul_pairs(uint32_t (&a)[S / TPI], const uint32_t *ys, const Modulus<S / TPI> &m,
+                                               uint32_t r) {
+  constexpr int L = S / TPI;
+  constexpr int kReduced = S / 2 - 2;  // steps between the first pair of rows and the last
+  constexpr int G = unrolled_steps<S, L, HOT>() > 0 ? unrolled_steps<S, L, HOT>() : 1;
+  constexpr int kHead = kReduced % G;
+  const uint2 *yp = reinterpret_cast<const uint2 *>(ys);
+  std::conditional_t<L % 2 == 0, PairSum<L, TPI>, OddPairSum<L, TPI>> t(r);
+  uint2 y = yp[0], next = yp[1];  // y is read one step ahead
+  t.start(a, y.x, y.y);
+#pragma unroll
+  for (int i = 1; i <= kHead; i++) {
+    y = next;
+    next = yp[i + 1];
+    t.template step<true>(a, y.x, y.y, m.f);
+  }
+  if constexpr (kReduced >= G) {
+#pragma unroll 1
+    for (int i0 = kHead + 1; i0 <= kReduced; i0 += G) {
+#pragma unroll
+      for (int i = 0; i < G; i++) {
+        y = next;
+        next = yp[i0 + i + 1];
+        t.template step<true>(a, y.x, y.y, m.f);
+      }
+    }
+  }
+  t.reduce(m);
+  t.template step<false>(a, next.x, next.y, m.f);
+  t.reduce(m);
+  const uint32_t pending = t.shift_out(a);
+  uint32_t topw = resolve<L, TPI>(a, pending, r);
+  topw = reduce_once<L, TPI>(a, topw, m.n, r);
+  if (m.tight) reduce_once<L, TPI>(a, topw, m.n, r);
+}
+
+template <int S, int TPI, bool HOT = false>
+__device__ __forceinline__ void mont(uint32_t (&a)[S / TPI], const uint32_t *ys, const Modulus<S / TPI> &m, uint32_t r) {
+  if constexpr (S / TPI > 1) {
+    mont_mul_pairs<S, TPI, HOT>(a, ys, m, r);
+  } else {
+    mont_mul_chain<S, TPI>(a, ys, m, r);
+  }
+}
+
+// a <- (a + b) mod N for a, b < N (distributed add, lookahead, one reduction).
+template <int L, int TPI>
+__device__ __forceinline__ void mod_add(uint32_t (&a)[L], const uint32_t (&b)[L], const uint32_t (&nn)[L], uint32_t r) {
+  uint32_t c;
+  add_cc(a[0], a[0], b[0]);
+#pragma unroll
+  for (int j = 1; j < L; j++) addc_cc(a[j], a[j], b[j]);
+  addc(c, 0u, 0u);
+  // c is this lane's carry into the next lane: reuse finalize, whose first
+  // step moves a lane's pending word into the next lane's limb 0.
+  finalize<L, TPI>(a, c, nn, r);
+}
+
 // Table of odd powers and the exponent walk.  On entry a = x in Montgomery
 // form; on exit a = x^E in Montgomery form.  tbl: the instance's odd-power
 // table (at least maxidx + 1 rows: the table size the schedule was built
 // for), ybuf: one row of this instance.  sched: steps of make_schedule()
-// (block-uniform).
+// (block-uniform).  Squarings and multiplications share one product in the
+// code, so that it can be unrolled whole.
 template <int S, int TPI>
 __device__ __forceinline__ void exp_window(uint32_t (&a)[S / TPI], uint32_t *tbl, uint32_t *ybuf,
                                            const uint32_t *__restrict__ sched, uint32_t nsteps, uint32_t maxidx,
-                                           const uint32_t (&nn)[S / TPI], uint32_t n0, uint32_t r) {
+                                           const Modulus<S / TPI> &m, uint32_t r) {
   constexpr int L = S / TPI;
   constexpr int ROW = Layout<S>::kRow;
   store_slice<L>(tbl, a, r);  // T[0] = x
   if (maxidx > 0) {
     store_slice<L>(ybuf, a, r);
-    __syncwarp();
-    mont<S, TPI>(a, ybuf, nn, n0, r);  // x^2
-    __syncwarp();
-    store_slice<L>(ybuf, a, r);
-    load_slice<L>(a, tbl, r);
-    __syncwarp();
+    // k = 0: x^2; k > 0: T[k] = T[k-1] x^2 = x^(2k+1)
 #pragma unroll 1
-    for (uint32_t k = 1; k <= maxidx; k++) {  // T[k] = T[k-1] x^2 = x^(2k+1)
-      mont<S, TPI>(a, ybuf, nn, n0, r);
-      store_slice<L>(tbl + k * ROW, a, r);
+    for (uint32_t k = 0; k <= maxidx; k++) {
+      __syncwarp();
+      mont<S, TPI>(a, ybuf, m, r);
+      if (k == 0) {
+        __syncwarp();
+        store_slice<L>(ybuf, a, r);
+        load_slice<L>(a, tbl, r);
+      } else {
+        store_slice<L>(tbl + k * ROW, a, r);
+      }
     }
     __syncwarp();
   }
   load_slice<L>(a, tbl + __ldg(sched) * ROW, r);
-#pragma unroll 1
-  for (uint32_t si = 1; si < nsteps; si++) {
-    const uint32_t step = __ldg(sched + si);
-    const uint32_t nsq = step >> 8, idx = step & 0xffu;
-#pragma unroll 1
-    for (uint32_t k = 0; k < nsq; k++) {
+  uint32_t si = 0, nsq = 0, idx = 0xffu;  // squarings and multiplication left of step si
+  for (;;) {
+    const uint32_t *y;
+    if (nsq > 0) {
+      nsq--;
       __syncwarp();
       store_slice<L>(ybuf, a, r);
       __syncwarp();
-      mont<S, TPI>(a, ybuf, nn, n0, r);
+      y = ybuf;
+    } else if (idx != 0xffu) {
+      y = tbl + idx * ROW;
+      idx = 0xffu;
+    } else {
+      if (++si >= nsteps) break;
+      const uint32_t step = __ldg(sched + si);
+      nsq = step >> 8;
+      idx = step & 0xffu;
+      continue;
     }
-    if (idx != 0xffu) mont<S, TPI>(a, tbl + idx * ROW, nn, n0, r);
+    mont<S, TPI, true>(a, y, m, r);
   }
 }
 

@@ -14,30 +14,20 @@ namespace dev {
 // the value in Montgomery form by R.  Two pieces take two products.
 template <int S, int TPI>
 __device__ __forceinline__ void crt_input(uint32_t (&a)[S / TPI], const uint32_t *c, bool active, int parts,
-                                          const uint32_t *sR2, const uint32_t *sR3, const uint32_t (&nn)[S / TPI],
-                                          uint32_t n0, uint32_t r) {
+                                          const uint32_t *sR2, const uint32_t *sR3, const Modulus<S / TPI> &m,
+                                          uint32_t r) {
   constexpr int L = S / TPI;
   uint32_t lo[L];
-  if (active) {
-    load_slice_global<L>(a, c + (parts - 1) * S, r);
-    load_slice_global<L>(lo, c + (parts - 2) * S, r);
-  } else {
 #pragma unroll
-    for (int j = 0; j < L; j++) lo[j] = a[j] = 0;
-  }
-  mont<S, TPI>(a, sR3, nn, n0, r);   // c_top R^2
-  mont<S, TPI>(lo, sR2, nn, n0, r);  // c_next R
-  mod_add<L, TPI>(a, lo, nn, r);           // (c_top R + c_next) R
-  for (int piece = parts - 3; piece >= 0; piece--) {
-    mont<S, TPI>(a, sR2, nn, n0, r);  // value * R, still in Montgomery form
-    if (active) {
-      load_slice_global<L>(lo, c + piece * S, r);
-    } else {
-#pragma unroll
-      for (int j = 0; j < L; j++) lo[j] = 0;
-    }
-    mont<S, TPI>(lo, sR2, nn, n0, r);
-    mod_add<L, TPI>(a, lo, nn, r);
+  for (int j = 0; j < L; j++) lo[j] = a[j] = 0;
+  if (active) load_slice_global<L>(a, c + (parts - 1) * S, r);
+#pragma unroll 1
+  for (int piece = parts - 2; piece >= 0; piece--) {
+    if (active) load_slice_global<L>(lo, c + piece * S, r);
+    // first c_top R^2, the Montgomery form of c_top R; then value * R
+    mont<S, TPI>(a, piece == parts - 2 ? sR3 : sR2, m, r);
+    mont<S, TPI>(lo, sR2, m, r);
+    mod_add<L, TPI>(a, lo, m.n, r);
   }
 }
 
@@ -101,7 +91,7 @@ __device__ __forceinline__ long long slot_chunk(const uint32_t *__restrict__ grp
 // schedules built for it.  grp: a key group table (explicit key indices), or
 // null for round robin.
 template <int S, int TPI, bool CRT, int NT = kThreads, int TABLE = kTableFull>
-__global__ void __launch_bounds__(NT) k_modexp(const KeyDev *__restrict__ keys, uint32_t K,
+__global__ void __launch_bounds__(NT, 1) k_modexp(const KeyDev *__restrict__ keys, uint32_t K,
                                                const uint32_t *__restrict__ in, uint32_t *__restrict__ out,
                                                long long n, int sel, int parts, const uint32_t *__restrict__ grp) {
   constexpr int L = S / TPI;
@@ -142,8 +132,9 @@ __global__ void __launch_bounds__(NT) k_modexp(const KeyDev *__restrict__ keys, 
   if (slot_chunk(grp, K, n, bc, (threadIdx.x / 32) * (32 / TPI)) < 0) return;
   const long long t = slot_chunk(grp, K, n, bc, g);
   const bool active = t >= 0;
-  uint32_t nn[L], a[L];
-  load_slice_global<L>(nn, M, r);
+  uint32_t a[L];
+  Modulus<L> m;
+  make_modulus<S, TPI>(m, M, n0, r);
   if (!CRT) {
     if (active) {
       load_slice_global<L>(a, in + t * W, r);
@@ -151,12 +142,12 @@ __global__ void __launch_bounds__(NT) k_modexp(const KeyDev *__restrict__ keys, 
 #pragma unroll
       for (int j = 0; j < L; j++) a[j] = 0;
     }
-    mont<S, TPI>(a, sR2, nn, n0, r);  // x R mod N
+    mont<S, TPI>(a, sR2, m, r);  // x R mod N
   } else {
-    crt_input<S, TPI>(a, in + t * W, active, parts, sR2, sR3, nn, n0, r);
+    crt_input<S, TPI>(a, in + t * W, active, parts, sR2, sR3, m, r);
   }
-  exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, nn, n0, r);
-  mont<S, TPI>(a, sOne, nn, n0, r);  // leave the Montgomery domain
+  exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, m, r);
+  mont<S, TPI>(a, sOne, m, r);  // leave the Montgomery domain
   if (active) {
     uint32_t *o = out + t * W + (CRT ? prime * S : 0) + r * L;
     if constexpr (L % 4 == 0) {

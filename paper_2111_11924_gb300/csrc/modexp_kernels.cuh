@@ -19,7 +19,7 @@ static __device__ __align__(16) uint32_t g_one_row[256] = {1u};
 // needs only its instances' tables, as many blocks fit per SM as for
 // k_modexp.
 template <int S, int TPI, bool CRT, int TABLE = kTableFull>
-__global__ void __launch_bounds__(kThreads) k_modexp_tasks(const BatchTask *__restrict__ tasks, int ntasks,
+__global__ void __launch_bounds__(kThreads, 1) k_modexp_tasks(const BatchTask *__restrict__ tasks, int ntasks,
                                                            int *__restrict__ counter) {
   constexpr int L = S / TPI;
   constexpr int IPW = 32 / TPI;
@@ -55,8 +55,9 @@ __global__ void __launch_bounds__(kThreads) k_modexp_tasks(const BatchTask *__re
     // The output address is formed before the exponentiation, so that only
     // this pointer (not the task's fields) stays live across it.
     uint32_t *const o = active ? tk.out + t * W + (CRT ? prime * S : 0) + r * L : nullptr;
-    uint32_t nn[L], a[L];
-    load_slice_global<L>(nn, M, r);
+    uint32_t a[L];
+    Modulus<L> m;
+    make_modulus<S, TPI>(m, M, n0, r);
     if (!CRT) {
       if (active) {
         load_slice_global<L>(a, tk.in + t * W, r);
@@ -64,12 +65,12 @@ __global__ void __launch_bounds__(kThreads) k_modexp_tasks(const BatchTask *__re
 #pragma unroll
         for (int j = 0; j < L; j++) a[j] = 0;
       }
-      mont<S, TPI>(a, sR2, nn, n0, r);
+      mont<S, TPI>(a, sR2, m, r);
     } else {
-      crt_input<S, TPI>(a, tk.in + t * W, active, parts, sR2, sR3, nn, n0, r);
+      crt_input<S, TPI>(a, tk.in + t * W, active, parts, sR2, sR3, m, r);
     }
-    exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, nn, n0, r);
-    mont<S, TPI>(a, sOne, nn, n0, r);
+    exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, m, r);
+    mont<S, TPI>(a, sOne, m, r);
     if (o) {
       if constexpr (L % 4 == 0) {
 #pragma unroll
@@ -102,8 +103,9 @@ __global__ void __launch_bounds__(kThreads) k_mulmod(const KeyDev *__restrict__ 
   for (int i = threadIdx.x; i < S; i += kThreads) sR2[i] = __ldg(kd.R2 + i);
   const long long t = first + (long long)g * K;
   const bool active = t < n;
-  uint32_t nn[L], a[L], b[L];
-  load_slice_global<L>(nn, kd.N, r);
+  uint32_t a[L], b[L];
+  Modulus<L> m;
+  make_modulus<S, TPI>(m, kd.N, kd.n0, r);
   if (active) {
     load_slice_global<L>(a, a_in + t * S, r);
     load_slice_global<L>(b, b_in + t * S, r);
@@ -113,8 +115,8 @@ __global__ void __launch_bounds__(kThreads) k_mulmod(const KeyDev *__restrict__ 
   }
   store_slice<L>(yrow, b, r);
   __syncthreads();
-  mont<S, TPI>(a, yrow, nn, kd.n0, r);
-  mont<S, TPI>(a, sR2, nn, kd.n0, r);
+  mont<S, TPI>(a, yrow, m, r);
+  mont<S, TPI>(a, sR2, m, r);
   if (active) {
     uint32_t *o = out + t * S + r * L;
 #pragma unroll
@@ -152,8 +154,9 @@ __global__ void __launch_bounds__(kThreads) k_crt_sum(const KeyDev *__restrict__
   const long long t = slot_chunk(grp, K, n, bc, g);
   const bool active = t >= 0;
   const int H = S / B;
-  uint32_t nn[L], acc[L], a[L];
-  load_slice_global<L>(nn, kd.N, r);
+  uint32_t acc[L], a[L];
+  Modulus<L> m;
+  make_modulus<S, TPI>(m, kd.N, kd.n0, r);
 #pragma unroll
   for (int j = 0; j < L; j++) acc[j] = 0;
   bool zero = false;
@@ -170,8 +173,8 @@ __global__ void __launch_bounds__(kThreads) k_crt_sum(const KeyDev *__restrict__
       for (int o = 1; o < TPI; o <<= 1) any |= __shfl_xor_sync(kFull, any, o, TPI);
     }
     zero = zero || any == 0;
-    mont<S, TPI>(a, smem + i * ROW, nn, kd.n0, r);  // m_i c_i mod N
-    mod_add<L, TPI>(acc, a, nn, r);
+    mont<S, TPI>(a, smem + i * ROW, m, r);  // m_i c_i mod N
+    mod_add<L, TPI>(acc, a, m.n, r);
   }
   if (active) {
     if (status && zero && r == 0) report(status, kStatusNotInvertible, t);
