@@ -419,15 +419,16 @@ int pmk_measure_imad_peak(pmk_ctx *ctx, double *mad_lo_per_clk_per_sm, double *s
  *          kernels (crt = 1) the limbs of one prime, nbits/(32 b) for a key
  *          with b primes (nbits/64 for an ordinary key).
  *   tpi:   lanes of a warp that hold one exponentiation (a power of two
- *          dividing 32 and the limb count); 0 restores the built-in default.
+ *          dividing 32 and the limb count); 0 restores the built-in choice,
+ *          made for each call from its number of exponentiations.
  *   form:  0, or 1 where pmk_list_kernel_configs lists it; both name the same
  *          kernel (1 was a second Montgomery product form).
  * Returns EUNSUPPORTED if that geometry is not compiled in.  Results are
  * bit-identical for every geometry; only speed differs.
  */
 int pmk_set_kernel_config(pmk_ctx *ctx, uint32_t limbs, int crt, uint32_t tpi, uint32_t form);
-/* The geometry the context currently uses for (limbs, crt).  EINVAL for a
- * NULL argument, EUNSUPPORTED if no kernel is compiled for (limbs, crt). */
+/* The geometry set for (limbs, crt), else the built-in one of calls that fill
+ * the GPU (smaller calls may take more lanes).  EINVAL for a NULL argument, EUNSUPPORTED if no kernel is compiled for (limbs, crt). */
 int pmk_get_kernel_config(const pmk_ctx *ctx, uint32_t limbs, int crt, uint32_t *tpi, uint32_t *form);
 /* Compiled geometries for (limbs, crt): writes up to `max` (tpi, form) pairs
  * and returns how many exist (a negative code on bad arguments).  Host only. */

@@ -88,6 +88,16 @@ pmk::KernelConfig cfg_for(const pmk_ctx *ctx, uint32_t limbs, bool crt) {
   return c;
 }
 
+// Kernel geometry of a call on n chunks: what the context sets for this width
+// and mode, else the choice for that many exponentiations.
+pmk::KernelConfig call_cfg(const pmk_ctx *ctx, const pmk_keyset *ks, bool crt, size_t n) {
+  const uint32_t limbs = ks->nbits / 32 / (crt ? ks->nprimes : 1u), key = limbs << 1 | (crt ? 1u : 0u);
+  if (ctx->cfg.count(key) || ctx->table.count(key)) return cfg_for(ctx, limbs, crt);
+  const long long K = ks->K;
+  return pmk::config_for_load(limbs, crt, pmk::Load{K * (crt ? ks->nprimes : 1u), ((long long)n + K - 1) / K, 0},
+                              ctx->sms);
+}
+
 // Whether any geometry for (limbs, crt) is compiled with the small table.
 bool small_table_available(uint32_t limbs, bool crt) {
   pmk::KernelConfig v[64];
@@ -217,7 +227,7 @@ int enqueue_encrypt(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *in, uint
   const uint32_t S = ks->nbits / 32;
   int rc = pmk::launch_range_check(ks->d_keys, ks->K, S, in, n, ctx->d_status, st, key_idx);
   if (rc == PMK_OK)
-    rc = pmk::launch_modexp(pmk::ExpMode::kEncrypt, S, cfg_for(ctx, S, false), ks->d_keys, ks->K, in, out, n, st,
+    rc = pmk::launch_modexp(pmk::ExpMode::kEncrypt, S, call_cfg(ctx, ks, false, n), ks->d_keys, ks->K, in, out, n, st,
                             ks->nprimes, groups, align);
   return rc;
 }
@@ -228,7 +238,7 @@ int enqueue_crt(pmk_ctx *ctx, const pmk_keyset *ks, pmk::ExpMode mode, const uin
                 cudaStream_t st, uint32_t *status_if_zero = nullptr, const uint32_t *groups = nullptr,
                 uint32_t align = pmk::kGroupAlign) {
   const uint32_t b = ks->nprimes, H = ks->nbits / 32 / b;
-  int rc = pmk::launch_modexp(mode, H, cfg_for(ctx, H, true), ks->d_keys, ks->K, in, out, n, st, b, groups, align);
+  int rc = pmk::launch_modexp(mode, H, call_cfg(ctx, ks, true, n), ks->d_keys, ks->K, in, out, n, st, b, groups, align);
   if (rc != PMK_OK) return rc;
   return pmk::launch_crt_sum(ks->nbits / 32, b, ks->d_keys, ks->K, out, n, st, status_if_zero, groups, align);
 }
@@ -240,7 +250,7 @@ int enqueue_decrypt(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *in, uint
   int rc = pmk::launch_range_check(ks->d_keys, ks->K, S, in, n, ctx->d_status, st, key_idx);
   if (rc != PMK_OK) return rc;
   if (!use_crt)
-    return pmk::launch_modexp(pmk::ExpMode::kDecrypt, S, cfg_for(ctx, S, false), ks->d_keys, ks->K, in, out, n, st,
+    return pmk::launch_modexp(pmk::ExpMode::kDecrypt, S, call_cfg(ctx, ks, false, n), ks->d_keys, ks->K, in, out, n, st,
                               ks->nprimes, groups, align);
   return enqueue_crt(ctx, ks, pmk::ExpMode::kCrtHalf, in, out, n, st, nullptr, groups, align);
 }
@@ -251,11 +261,11 @@ int enqueue_decrypt(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *in, uint
 // and can stack three working blocks on an SM where round robin puts two:
 // 1.5x the time at 4096 bits and 1 MiB, measured).  0 when a width has no
 // kernel.
-uint32_t group_align(const pmk_ctx *ctx, const pmk_keyset *ks, bool use_crt) {
+uint32_t group_align(const pmk_ctx *ctx, const pmk_keyset *ks, bool use_crt, size_t n) {
   const uint32_t S = ks->nbits / 32;
-  if (!use_crt) return pmk::modexp_block_instances(S, cfg_for(ctx, S, false), false);
+  if (!use_crt) return pmk::modexp_block_instances(S, call_cfg(ctx, ks, false, n), false);
   const uint32_t H = S / ks->nprimes;
-  return std::max(pmk::modexp_block_instances(H, cfg_for(ctx, H, true), true), pmk::crt_sum_block_instances(S));
+  return std::max(pmk::modexp_block_instances(H, call_cfg(ctx, ks, true, n), true), pmk::crt_sum_block_instances(S));
 }
 
 // Explicit key indices: check them on the host side of the call, then build
@@ -297,6 +307,10 @@ int pmk_create(pmk_ctx **out, int cuda_device) {
   ctx->device = cuda_device;
   DeviceGuard g(cuda_device);
   if (!g.ok()) {
+    delete ctx;
+    return PMK_ECUDA;
+  }
+  if (cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, cuda_device) != cudaSuccess) {
     delete ctx;
     return PMK_ECUDA;
   }
@@ -668,7 +682,7 @@ int pmk_encrypt_chunks(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *d_in,
   if (!g.ok()) return PMK_ECUDA;
   cudaStream_t st = as_stream(stream);
   const uint32_t *groups = nullptr;
-  const uint32_t align = d_key_idx ? group_align(ctx, ks, false) : pmk::kGroupAlign;
+  const uint32_t align = d_key_idx ? group_align(ctx, ks, false, n_chunks) : pmk::kGroupAlign;
   rc = key_groups_for(ctx, ks, d_key_idx, n_chunks, st, align, &groups);
   if (rc == PMK_OK) rc = enqueue_encrypt(ctx, ks, d_in, d_out, n_chunks, st, d_key_idx, groups, align);
   if (d_key_idx) release(ctx->grp, st);
@@ -687,7 +701,7 @@ int pmk_decrypt_chunks(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *d_in,
   if (!g.ok()) return PMK_ECUDA;
   cudaStream_t st = as_stream(stream);
   const uint32_t *groups = nullptr;
-  const uint32_t align = d_key_idx ? group_align(ctx, ks, use_crt != 0) : pmk::kGroupAlign;
+  const uint32_t align = d_key_idx ? group_align(ctx, ks, use_crt != 0, n_chunks) : pmk::kGroupAlign;
   rc = key_groups_for(ctx, ks, d_key_idx, n_chunks, st, align, &groups);
   if (rc == PMK_OK) rc = enqueue_decrypt(ctx, ks, d_in, d_out, n_chunks, use_crt, st, d_key_idx, groups, align);
   if (d_key_idx) release(ctx->grp, st);
@@ -747,7 +761,7 @@ int pmk_decrypt_blinded(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *d_cs
   if (rc != PMK_OK) return rc;
   // m = x^d
   if (!use_crt)
-    return pmk::launch_modexp(pmk::ExpMode::kDecrypt, S, cfg_for(ctx, S, false), ks->d_keys, ks->K, d_m, d_m,
+    return pmk::launch_modexp(pmk::ExpMode::kDecrypt, S, call_cfg(ctx, ks, false, n_chunks), ks->d_keys, ks->K, d_m, d_m,
                               n_chunks, st);
   rc = acquire(ctx->b, n_chunks * S * 4, st);
   uint32_t *x = static_cast<uint32_t *>(ctx->b.ptr);

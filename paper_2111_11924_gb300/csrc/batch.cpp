@@ -64,6 +64,37 @@ void release(pmk_batch *b) {
   cudaFree(b->d_counters);
 }
 
+// The lane counts of the jobs with a launch of their own, where the context
+// sets none.  Their launches run at the same time, so a job's load is its own
+// exponentiations and, beside them, those of every other job: all that last
+// as long as the job's own, and of a shorter kind the share of the time that
+// they last (an encryption is over at once).
+void choose_lanes(const pmk_ctx *ctx, const std::vector<pmk::PlanJob> &jobs, std::vector<pmk::PlanDirect> &direct) {
+  struct Work {
+    double count, length;  // exponentiations, and the multiply-adds of one
+    uint32_t limbs;
+    bool crt;
+  };
+  std::vector<Work> work;
+  for (const pmk::PlanDirect &d : direct) {
+    const pmk::PlanJob &j = jobs[d.job];
+    const bool crt = j.op == PMK_OP_DECRYPT_CRT;
+    const double bits = j.op == PMK_OP_ENCRYPT ? 17.0 : 32.0 * d.limbs;  // products of one exponentiation, about
+    work.push_back(Work{(double)j.n_chunks * (crt ? j.nprimes : 1u), bits * d.limbs * d.limbs, d.limbs, crt});
+  }
+  for (size_t i = 0; i < direct.size(); i++) {
+    const pmk::PlanJob &j = jobs[direct[i].job];
+    const uint32_t key = work[i].limbs << 1 | (work[i].crt ? 1u : 0u);
+    if (ctx->cfg.count(key) || ctx->table.count(key)) continue;
+    double beside = 0;
+    for (size_t k = 0; k < work.size(); k++)
+      if (k != i) beside += work[k].count * std::min(1.0, work[k].length / work[i].length);
+    const long long K = j.K, rows = K * (work[i].crt ? j.nprimes : 1u);
+    direct[i].cfg = pmk::config_for_load(work[i].limbs, work[i].crt,
+                                         pmk::Load{rows, ((long long)j.n_chunks + K - 1) / K, (long long)beside}, ctx->sms);
+  }
+}
+
 int plan_and_capture(pmk_ctx *ctx, const pmk_job *jobs, size_t n_jobs, pmk_batch *b) {
   std::vector<pmk::PlanJob> plan_jobs(n_jobs);
   for (size_t j = 0; j < n_jobs; j++) {
@@ -86,8 +117,8 @@ int plan_and_capture(pmk_ctx *ctx, const pmk_job *jobs, size_t n_jobs, pmk_batch
   std::vector<pmk::PlanDirect> direct;  // jobs with a grid launch of their own
   int rc = pmk::plan_batch(plan_jobs, config, resident, ctx->batch_direct_max, planned, direct);
   if (rc != PMK_OK) return rc;
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device) != cudaSuccess) return PMK_ECUDA;
+  const int sms = ctx->sms;
+  choose_lanes(ctx, plan_jobs, direct);
   std::vector<Group> groups(planned.size());
   std::vector<pmk::BatchTask> all;
   for (size_t gi = 0; gi < planned.size(); gi++) {

@@ -1,5 +1,5 @@
 // Instantiations and launcher of the fused blinded CRT decryption
-// (modexp_blind.cuh): one geometry per prime limb count, the CRT default.
+// (modexp_blind.cuh).
 #include "modexp_blind.cuh"
 #include "modexp_kernels.cuh"
 
@@ -18,22 +18,14 @@ BlindEntry make_blind() {
                     dev::modexp_smem_bytes<S>(TPI, NT)};
 }
 
-// Throughput geometries (the CRT defaults), then geometries with more lanes
-// per instance for small batches (a shorter chain per exponentiation).
+// For each prime width the throughput geometry (the CRT default) first, then
+// those with more lanes per instance.
 const BlindEntry *blind_entries(int *count) {
   static const BlindEntry entries[] = {
-      make_blind<2, 2>(),  make_blind<4, 2>(),  make_blind<8, 2>(),
-      make_blind<16, 2>(), make_blind<32, 4, 64>(), make_blind<48, 8>(),
-      make_blind<64, 8>(), make_blind<96, 8>(),  make_blind<128, 16>(),
-  };
-  *count = (int)(sizeof(entries) / sizeof(entries[0]));
-  return entries;
-}
-
-const BlindEntry *blind_entries_latency(int *count) {
-  static const BlindEntry entries[] = {
-      make_blind<16, 8>(),  make_blind<32, 16>(), make_blind<48, 16>(),
-      make_blind<64, 32>(), make_blind<96, 16>(), make_blind<128, 32>(),
+      make_blind<2, 2>(),   make_blind<4, 2>(),   make_blind<8, 2>(),   make_blind<16, 2>(),  make_blind<16, 8>(),
+      make_blind<32, 4, 64>(), make_blind<32, 8>(), make_blind<32, 16>(), make_blind<48, 8>(), make_blind<48, 16>(),
+      make_blind<64, 8>(),  make_blind<64, 16>(), make_blind<64, 32>(), make_blind<96, 8>(),  make_blind<96, 16>(),
+      make_blind<128, 16>(), make_blind<128, 32>(),
   };
   *count = (int)(sizeof(entries) / sizeof(entries[0]));
   return entries;
@@ -54,17 +46,20 @@ int launch_blind_crt(uint32_t prime_limbs, uint32_t parts, const KeyDev *keys, u
   if (n == 0) return PMK_OK;
   if (parts < 2 || parts > (uint32_t)kMaxPrimes || (unsigned long long)K * parts > 65535ull) return PMK_EINVAL;
   int cnt = 0, dev = 0, sms = 0;
-  const BlindEntry *list = blind_entries(&cnt), *e = nullptr;
-  for (int i = 0; i < cnt; i++)
-    if (list[i].limbs == (int)prime_limbs) e = &list[i];
-  if (!e) return PMK_EUNSUPPORTED;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return PMK_ECUDA;
-  if ((long long)n * parts < 16LL * sms) {  // too few exponentiations to fill the GPU: shorten each one
-    const BlindEntry *lat = blind_entries_latency(&cnt);
-    for (int i = 0; i < cnt; i++)
-      if (lat[i].limbs == (int)prime_limbs) e = &lat[i];
+  const BlindEntry *list = blind_entries(&cnt), *e = nullptr;
+  const Load load{(long long)K * parts, ((long long)n + K - 1) / K, 0};
+  long long least = 0;
+  for (int i = 0; i < cnt; i++) {  // the lane count estimated fastest, as config_for_load
+    if (list[i].limbs != (int)prime_limbs) continue;
+    const long long c = product_clocks(list[i].limbs, list[i].tpi, load, sms);
+    if (!e || c < least) {
+      e = &list[i];
+      least = c;
+    }
   }
+  if (!e) return PMK_EUNSUPPORTED;
   int rc = configure_smem(e->fn, e->smem);
   if (rc != PMK_OK) return rc;
   const long long per_key = ((long long)n + K - 1) / K;

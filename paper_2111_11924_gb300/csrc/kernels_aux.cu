@@ -335,10 +335,15 @@ std::vector<ModexpEntry> entries(bool crt) {
   return v;
 }
 
-const ModexpEntry *find_exact(uint32_t limbs, KernelConfig cfg, bool crt) {
+const std::vector<ModexpEntry> &built(bool crt) {
   static const std::vector<ModexpEntry> full = entries(false), residue = entries(true);
-  for (const ModexpEntry &e : crt ? residue : full)
-    if (e.limbs == (int)limbs && e.tpi == (int)cfg.tpi && cfg.form < 2 && (e.forms >> cfg.form & 1u) && e.table == cfg.table) return &e;
+  return crt ? residue : full;
+}
+
+const ModexpEntry *find_exact(uint32_t limbs, KernelConfig cfg, bool crt) {
+  for (const ModexpEntry &e : built(crt))
+    if (e.limbs == (int)limbs && e.tpi == (int)cfg.tpi && cfg.form < 2 && (e.forms >> cfg.form & 1u) && e.table == cfg.table)
+      return &e;
   return nullptr;
 }
 
@@ -536,10 +541,45 @@ KernelConfig default_config(uint32_t limbs, bool crt) {
   return c;
 }
 
+// A product is S / 2 steps; a step's clocks grow with the limbs per lane L
+// and the warps w that share a scheduler.  Lines through the measured clocks
+// per step (64 limbs on 2, 4, 8 limbs per lane): one warp 78 / 120 / 214,
+// two 118 / 178 / 308, each further one 44 / 86 / 150.  One warp alone issues
+// a wide multiply-add per 6.6 clocks, so w = 2 costs much less than twice.
+long long product_clocks(int limbs, int tpi, const Load &load, int sms) {
+  const long long L = limbs / tpi, ipw = 32 / tpi;
+  const long long warps = load.rows * ((load.per_row + ipw - 1) / ipw) + (load.beside + ipw - 1) / ipw;
+  const long long w = (warps + 4LL * sms - 1) / (4LL * sms);
+  return limbs / 2 * (w <= 1 ? 30 + 23 * L : 52 + 32 * L + (w - 2) * (8 + 19 * L));
+}
+
+// More lanes shorten one exponentiation and cost more in total, so they pay
+// while the GPU has schedulers to spare.  Measured, ms by lanes: full d at
+// 2048 bits, 403 chunks 8.06 (8 lanes) / 4.55 (16) / 3.09 (32), 1,024 chunks
+// 8.07 / 4.56 / 4.46, 2,056 chunks 8.07 / 6.61 / 8.18, 4,113 chunks 11.7 / 12.7
+// / 13.9; CRT at 3072 bits, 685 chunks 3.70 (8) / 3.41 (16), 6,000 chunks 12.7
+// / 14.9.  Fewer lanes than the default are not considered: their tables
+// leave too few exponentiations on an SM.
+KernelConfig config_for_load(uint32_t limbs, bool crt, const Load &load, int sms) {
+  KernelConfig best = default_config(limbs, crt);
+  if (best.tpi == 0 || sms <= 0) return best;
+  const int base = (int)best.tpi;
+  long long least = product_clocks((int)limbs, base, load, sms);
+  for (const ModexpEntry &e : built(crt)) {
+    if (e.limbs != (int)limbs || e.table != kTableFull || e.tpi <= base) continue;
+    const long long c = product_clocks((int)limbs, e.tpi, load, sms);
+    if (c < least) {
+      least = c;
+      best = KernelConfig{(uint32_t)e.tpi, e.forms & kForm0 ? 0u : 1u};
+    }
+  }
+  return best;
+}
+
 int list_configs(uint32_t limbs, bool crt, KernelConfig *out, int max) {
   int k = 0;
   for (uint32_t form = 0; form < 2; form++)
-    for (const ModexpEntry &e : entries(crt)) {
+    for (const ModexpEntry &e : built(crt)) {
       // geometries; small-table twins are not listed
       if (e.limbs != (int)limbs || e.table != kTableFull || !(e.forms >> form & 1u)) continue;
       if (k < max && out) out[k] = KernelConfig{(uint32_t)e.tpi, form};

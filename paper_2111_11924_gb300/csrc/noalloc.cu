@@ -97,12 +97,18 @@ extern "C" int pmk_decrypt_message_host_noalloc(const pmk_keyset *ks, const uint
       rc = PMK_ECUDA;
       break;
     }
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ks->device) != cudaSuccess) {
+      rc = PMK_ECUDA;
+      break;
+    }
+    const long long K = ks->K, per_key = ((long long)n_chunks + K - 1) / K;
     rc = launch_range_check(ks->d_keys, ks->K, S, d_cipher, n_chunks, d_status, st);
     if (rc == PMK_OK && !use_crt)
-      rc = launch_modexp(ExpMode::kDecrypt, S, default_config(S, false), ks->d_keys, ks->K, d_cipher, d_plain, n_chunks, st);
+      rc = launch_modexp(ExpMode::kDecrypt, S, config_for_load(S, false, Load{K, per_key, 0}, sms), ks->d_keys, ks->K, d_cipher, d_plain, n_chunks, st);
     if (rc == PMK_OK && use_crt) {
-      rc = launch_modexp(ExpMode::kCrtHalf, H, default_config(H, true), ks->d_keys, ks->K, d_cipher, d_plain, n_chunks,
-                         st, B);
+      rc = launch_modexp(ExpMode::kCrtHalf, H, config_for_load(H, true, Load{K * B, per_key, 0}, sms), ks->d_keys, ks->K,
+                         d_cipher, d_plain, n_chunks, st, B);
       if (rc == PMK_OK)
         rc = launch_crt_sum(S, B, ks->d_keys, ks->K, d_plain, n_chunks, st);
     }

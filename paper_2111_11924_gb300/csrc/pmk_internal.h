@@ -224,6 +224,18 @@ bool modexp_small_table_built(uint32_t limbs, KernelConfig cfg, bool crt);
 int launch_modexp_naive(bool enc, uint32_t limbs, const KeyDev *keys, uint32_t K, const uint32_t *in, uint32_t *out,
                         size_t n, cudaStream_t st);
 KernelConfig default_config(uint32_t limbs, bool crt);  // tpi == 0: limb count not built
+// The exponentiations of one launch: `rows` (key, prime) pairs with `per_row`
+// chunks each, and `beside` of the same width that other launches run on the
+// GPU meanwhile.
+struct Load {
+  long long rows, per_row, beside;
+};
+// Estimated clocks of one Montgomery product of S limbs on tpi lanes under
+// that load on `sms` multiprocessors (for comparing lane counts).
+long long product_clocks(int limbs, int tpi, const Load &load, int sms);
+// The geometry of a call whose context sets none: default_config, or more
+// lanes where that is estimated to finish sooner.
+KernelConfig config_for_load(uint32_t limbs, bool crt, const Load &load, int sms);
 int list_configs(uint32_t limbs, bool crt, KernelConfig *out, int max);
 // Persistent batch kernel for (limbs, cfg, crt): `blocks` x 128 threads
 // drain tasks[0..ntasks) through *counter (which must start at zero).
@@ -272,6 +284,7 @@ constexpr size_t kDirectMaxJobs = 256;
 // Context: one device, its status record, staging and kernel geometry choices.
 struct pmk_ctx {
   int device = 0;
+  int sms = 0;                             // multiprocessors of the device
   uint32_t *d_status = nullptr;            // status record: error bits, smallest failing chunk
   pmk::Staging msg, a, b;                  // staging of the *_host calls and the blinded CRT path
   pmk::Staging grp;                        // key-group table of calls with explicit key indices

@@ -496,7 +496,7 @@ class Context:
         return {"mad_lo_per_clk_per_sm": m.value, "sm_mhz": mhz.value, "num_sms": sms.value}
 
     def set_kernel_config(self, limbs: int, crt: bool, tpi: int, form: int = 0) -> None:
-        """Lanes per instance and Montgomery form for (limbs, crt); tpi = 0 restores the default."""
+        """Lanes per instance and Montgomery form for (limbs, crt); tpi = 0 restores the built-in choice (by call size)."""
         _check(load_library().pmk_set_kernel_config(self.handle, limbs, int(crt), tpi, form), "pmk_set_kernel_config")
 
     def set_kernel_window(self, limbs: int, crt: bool, max_window: int) -> None:
@@ -539,11 +539,14 @@ class Context:
 
     def copy_kernel_configs_from(self, other: "Context", keysets: dict) -> None:
         """Take other's kernel geometry and window bound for every limb count
-        the key sets use (full width and CRT residues)."""
+        the key sets use (full width and CRT residues).  A width where other
+        has the built-in geometry stays unset, so that each call's size picks
+        its lanes."""
         for ks in keysets.values():
             for limbs, crt in ((ks.nbits // 32, False), (ks.nbits // 32 // ks.nprimes, True)):
-                tpi, form = other.get_kernel_config(limbs, crt)
-                self.set_kernel_config(limbs, crt, tpi, form)
+                cfg = other.get_kernel_config(limbs, crt)
+                if cfg != self.get_kernel_config(limbs, crt):
+                    self.set_kernel_config(limbs, crt, *cfg)
                 self.set_kernel_window(limbs, crt, other.get_kernel_window(limbs, crt))
 
     def get_kernel_config(self, limbs: int, crt: bool) -> tuple:
