@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kThreads) k_mulmod(const KeyDev *__restrict__ 
                                                      long long n) {
   constexpr int L = S / TPI;
   constexpr int IPB = kThreads / TPI;
-  constexpr int ROW = Layout<S>::kRow;
+  constexpr int ROW = Layout<S>::kLoneRow;
   extern __shared__ __align__(16) uint32_t smem[];
   const uint32_t r = threadIdx.x % TPI, g = threadIdx.x / TPI;
   uint32_t *sR2 = smem, *yrow = smem + (1 + g) * ROW;
@@ -212,11 +212,9 @@ struct ModexpEntry {
 enum : uint32_t { kForm0 = 1u, kForm01 = 3u };
 
 // NT: block size of the one-launch-per-call kernel.  64 for 32 limbs at 4
-// lanes: a 128-thread block (32 instance tables, 78 KB) leaves two per SM
-// and much shared memory unused, 64-thread blocks fit five (64 -> 80
-// instances per SM): 3.4% faster CRT decryption at 2048 bits and 100 MiB.
-// Other geometries measured no gain or a loss (64 limbs at 4 lanes: 12%
-// slower at 1 MiB) and keep 128.
+// lanes, where a smaller block leaves less of an SM's shared memory unused
+// and a key's last block smaller; other geometries measured no gain or a loss
+// (64 limbs at 4 lanes: 12% slower at 1 MiB) and keep 128.
 template <int S, int TPI, bool CRT, int NT = dev::kThreads, int TABLE = kTableFull>
 ModexpEntry make_entry(uint32_t forms) {
   constexpr size_t warp_area = (size_t)(32 / TPI) * dev::Layout<S>::inst(dev::table_rows(TABLE));
@@ -248,7 +246,7 @@ struct MulmodEntry {
 template <int S, int TPI>
 MulmodEntry make_mulmod() {
   return MulmodEntry{S, TPI, reinterpret_cast<const void *>(&dev::k_mulmod<S, TPI>),
-                     sizeof(uint32_t) * (size_t)(1 + dev::kThreads / TPI) * dev::Layout<S>::kRow};
+                     sizeof(uint32_t) * (size_t)(1 + dev::kThreads / TPI) * dev::Layout<S>::kLoneRow};
 }
 const MulmodEntry *mulmod_entries(int *count);
 
