@@ -588,7 +588,10 @@ int list_configs(uint32_t limbs, bool crt, KernelConfig *out, int max) {
   return k;
 }
 
-// Raise a kernel's dynamic shared-memory limit once per device.
+// Raise a kernel's dynamic shared-memory limit once per device, and ask for
+// the same split of L1 for all: an SM changes its split only when it is idle,
+// so kernels with different ones do not share it (a batch of 24 messages
+// through the task queues: 40 instead of 18 ms).
 int configure_smem(const void *fn, size_t bytes) {
   static std::mutex mu;
   static std::set<std::pair<const void *, int>> done;
@@ -596,7 +599,9 @@ int configure_smem(const void *fn, size_t bytes) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return PMK_ECUDA;
   if (!done.count({fn, dev})) {
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
+            cudaSuccess)
       return PMK_ECUDA;
     done.insert({fn, dev});
   }

@@ -211,10 +211,14 @@ struct ModexpEntry {
 
 enum : uint32_t { kForm0 = 1u, kForm01 = 3u };
 
-// NT: block size of the one-launch-per-call kernel.  64 for 32 limbs at 4
-// lanes, where a smaller block leaves less of an SM's shared memory unused
-// and a key's last block smaller; other geometries measured no gain or a loss
-// (64 limbs at 4 lanes: 12% slower at 1 MiB) and keep 128.
+// NT: block size of the one-launch-per-call kernel.  32 where many lanes serve
+// few exponentiations: the warps of a key's last block that have none end at
+// once, and since a block's first warp always goes to the same scheduler,
+// 128-thread blocks left the schedulers uneven (64 limbs on 32 lanes, 1,024
+// chunks: 4.46 instead of 4.26 ms; twelve jobs of 78 chunks side by side, 48
+// limbs on 16 lanes: 4.96 instead of 3.61 ms).  64 for 32 limbs at 4 lanes,
+// where a smaller block leaves less of an SM's shared memory unused; the
+// other throughput geometries measured no gain or a loss and keep 128.
 template <int S, int TPI, bool CRT, int NT = dev::kThreads, int TABLE = kTableFull>
 ModexpEntry make_entry(uint32_t forms) {
   constexpr size_t warp_area = (size_t)(32 / TPI) * dev::Layout<S>::inst(dev::table_rows(TABLE));

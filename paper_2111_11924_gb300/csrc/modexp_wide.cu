@@ -11,13 +11,13 @@ const ModexpEntry *modexp_entries_wide(int *count) {
       make_entry<256, 16, false>(kForm01),
       make_entry<256, 32, false>(kForm0),
       make_entry<96, 8, true>(kForm0),
-      make_entry<96, 16, true>(kForm01),
+      make_entry<96, 16, true, 32>(kForm01),
       make_entry<128, 16, true>(kForm01),
-      make_entry<96, 16, false>(kForm01),
-      make_entry<48, 16, true>(kForm0),
-      make_entry<128, 32, false>(kForm0),
+      make_entry<96, 16, false, 32>(kForm01),
+      make_entry<48, 16, true, 32>(kForm0),
+      make_entry<128, 32, false, 32>(kForm0),
       make_entry<192, 32, false>(kForm0),
-      make_entry<64, 32, false>(kForm0),
+      make_entry<64, 32, false, 32>(kForm0),
   };
   *count = (int)(sizeof(entries) / sizeof(entries[0]));
   return entries;
