@@ -117,7 +117,7 @@ size_t push(std::vector<uint32_t> &blob, const std::vector<uint32_t> &v) {
 int upload(pmk_keyset *ks) {
   std::vector<uint32_t> blob;
   struct Offs {
-    size_t N, R2, se[2], sd[2], P[pmk::kMaxPrimes], R2h[pmk::kMaxPrimes], R3h[pmk::kMaxPrimes],
+    size_t N, R2, Re, se[2], sd[2], P[pmk::kMaxPrimes], R2h[pmk::kMaxPrimes], R3h[pmk::kMaxPrimes],
         sh[2][pmk::kMaxPrimes], shi[2][pmk::kMaxPrimes], cs[pmk::kMaxPrimes], sb[pmk::kMaxPrimes], el, dl;
   };
   std::vector<Offs> offs(ks->K);
@@ -126,6 +126,7 @@ int upload(pmk_keyset *ks) {
     Offs &o = offs[k];
     o.N = push(blob, h.N);
     o.R2 = push(blob, h.R2);
+    o.Re = push(blob, h.Re);
     for (int t = 0; t < 2; t++) {
       o.se[t] = push(blob, h.sched_e[t].steps);
       o.sd[t] = push(blob, h.sched_d[t].steps);
@@ -161,6 +162,7 @@ int upload(pmk_keyset *ks) {
     d = KeyDev{};
     d.N = b + o.N;
     d.R2 = b + o.R2;
+    d.Re = b + o.Re;
     d.e_limbs = b + o.el;
     d.d_limbs = b + o.dl;
     d.n0 = h.n0;

@@ -371,6 +371,13 @@ void finish_key(uint32_t nbits, u64 e, const std::vector<std::vector<u64>> &r, H
   }
   // CRT recombination rows c_i R mod N, c_i = (N / r_i) ((N / r_i)^-1 mod r_i)
   const Mont mN(N);
+  {  // R^e mod N
+    std::vector<u64> one(s / 2, 0), R(s / 2), Re(s / 2);
+    one[0] = 1;
+    mN.to_mont(R.data(), one.data());
+    mN.pow(Re.data(), R.data(), &e, 1);
+    k.Re = to32(Re, s);
+  }
   for (int i = 0; i < b; i++) {
     const Mont mt(r[i]);
     std::vector<u64> others, acc(n), t(n), x(n), inv(n), rm2(r[i]);

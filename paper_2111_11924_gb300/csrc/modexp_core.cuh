@@ -739,7 +739,7 @@ __device__ __forceinline__ void mod_add(uint32_t (&a)[L], const uint32_t (&b)[L]
 }
 
 // Table of odd powers and the exponent walk.  On entry a = x in Montgomery
-// form; on exit a = x^E in Montgomery form.  tbl: the instance's odd-power
+// form; on exit a = x^E in Montgomery form (of any x < N: x^E R^-(E-1) mod N).  tbl: the instance's odd-power
 // table (at least maxidx + 1 rows: the table size the schedule was built
 // for), ybuf: one row of this instance.  sched: steps of make_schedule()
 // (block-uniform).  Squarings and multiplications share one product in the

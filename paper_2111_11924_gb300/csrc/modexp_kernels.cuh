@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_modexp_tasks(const BatchTask *_
     const uint32_t nsteps = CRT ? kd.nsteps_h[TABLE][prime] : (enc ? kd.nsteps_e[TABLE] : kd.nsteps_d[TABLE]);
     const uint32_t maxidx = CRT ? kd.maxidx_h[TABLE][prime] : (enc ? kd.maxidx_e[TABLE] : kd.maxidx_d[TABLE]);
     const uint32_t n0 = CRT ? kd.n0h[prime] : kd.n0;
-    const uint32_t *sR2 = R2, *sR3 = CRT ? kd.R3h[prime] : R2, *sOne = g_one_row;
+    const uint32_t *sR2 = R2, *sR3 = CRT ? kd.R3h[prime] : R2, *sLast = !CRT && enc ? kd.Re : g_one_row;
     const bool active = (int)g < tk.count;
     const long long t = tk.first + (long long)g * tk.stride;
     // The output address is formed before the exponentiation, so that only
@@ -65,12 +65,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_modexp_tasks(const BatchTask *_
 #pragma unroll
         for (int j = 0; j < L; j++) a[j] = 0;
       }
-      mont<S, TPI>(a, sR2, m, r);
+      if (enc) {
+        reduce_once<L, TPI>(a, 0u, m.n, r);
+      } else {
+        mont<S, TPI>(a, sR2, m, r);
+      }
     } else {
       crt_input<S, TPI>(a, tk.in + t * W, active, parts, sR2, sR3, m, r);
     }
     exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, m, r);
-    mont<S, TPI>(a, sOne, m, r);
+    mont<S, TPI>(a, sLast, m, r);
     if (o) {
       if constexpr (L % 4 == 0) {
 #pragma unroll

@@ -110,6 +110,7 @@ struct HostKey {
   // Montgomery data, R = 2^(32 s) for N and R_h = 2^(32 h) for the primes.
   uint32_t n0 = 0, n0h[kMaxPrimes] = {};               // -M^-1 mod 2^32
   std::vector<uint32_t> R2;                            // R^2 mod N
+  std::vector<uint32_t> Re;                            // R^e mod N
   std::vector<uint32_t> R2h[kMaxPrimes], R3h[kMaxPrimes];  // R_h^2, R_h^3 mod r_i
   // Exponent schedules per table size (kTableFull, kTableSmall): e, d,
   // d mod (r_i - 1) and r_i - 2 (Fermat inverses mod r_i).
@@ -125,6 +126,7 @@ struct KeyDev {
   // [kTableFull] or [kTableSmall].
   const uint32_t *N;
   const uint32_t *R2;
+  const uint32_t *Re;
   const uint32_t *sched_e[2], *sched_d[2];
   const uint32_t *P[kMaxPrimes];
   const uint32_t *R2h[kMaxPrimes];

@@ -70,3 +70,33 @@ def test_all_ones_moduli_every_geometry(nbits, crt):
         ctx.check()
         ks.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("nbits", (128, 512, 1024, 2048))
+def test_chunks_not_below_the_modulus(nbits):
+    """A chunk >= N is reported and still gives its residue's power, per call
+    and through the task queues, for every geometry."""
+    import torch
+
+    import paper_2111_11924_gb300 as P
+    from paper_2111_11924_gb300 import pmkrsa
+
+    ctx = P.Context(0)
+    ks = ctx.keygen(2, nbits, 65537, 23)
+    Ns = [int.from_bytes(r.tobytes(), "little") for r in ks.export()["N"]]
+    top = (1 << nbits) - 1
+    m = [x for pair in zip(*((N, N + 1, top, N - 1, 0, 3) for N in Ns)) for x in pair]  # chunk t under key t mod 2
+    d_m = torch.from_numpy(_limbs(m, nbits).view(np.int32)).cuda()
+    want = torch.from_numpy(_limbs([pow(x, 65537, Ns[t % 2]) for t, x in enumerate(m)], nbits).view(np.int32)).cuda()
+    for tpi, form in P.kernel_configs(nbits // 32, False):
+        ctx.set_kernel_config(nbits // 32, False, tpi, form)
+        assert torch.equal(ctx.encrypt_chunks(ks, d_m), want), (tpi, form)
+        assert ctx.status() == pmkrsa.PMK_ERANGE
+        for direct in (256, 0):
+            out = torch.zeros_like(d_m)
+            ctx.set_batch_direct_max(direct)
+            batch = ctx.batch([(ks, d_m, out, pmkrsa.OP_ENCRYPT)])
+            batch.launch()
+            assert ctx.status() == pmkrsa.PMK_ERANGE
+            assert torch.equal(out, want), (tpi, form, direct)
+    ctx.close()
