@@ -153,8 +153,7 @@ __global__ void __launch_bounds__(NT, 1) k_modexp(const KeyDev *__restrict__ key
   } else {
     crt_input<S, TPI>(a, in + t * W, active, parts, sR2, sR3, m, r);
   }
-  exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, m, r);
-  mont<S, TPI>(a, sLast, m, r);  // leave the Montgomery domain
+  exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, sLast, m, r);  // and leave the Montgomery domain
   if (active) {
     uint32_t *o = out + t * W + (CRT ? prime * S : 0) + r * L;
     if constexpr (L % 4 == 0) {

@@ -73,8 +73,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_modexp_tasks(const BatchTask *_
     } else {
       crt_input<S, TPI>(a, tk.in + t * W, active, parts, sR2, sR3, m, r);
     }
-    exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, m, r);
-    mont<S, TPI>(a, sLast, m, r);
+    exp_window<S, TPI>(a, tbl, ybuf, sched, nsteps, maxidx, sLast, m, r);
     if (o) {
       if constexpr (L % 4 == 0) {
 #pragma unroll
