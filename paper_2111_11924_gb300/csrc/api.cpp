@@ -220,18 +220,14 @@ int check_chunk_call(const pmk_ctx *ctx, const pmk_keyset *ks, const void *in, c
   return PMK_OK;
 }
 
-// key_idx / groups / align: explicit key indices and their key-group table
+// groups / align: the key-group table of explicit key indices
 // (launch_key_groups, with that alignment), or NULL for round robin (chunk
-// t -> key t mod K).
+// t -> key t mod K).  The exponentiation itself checks the range of a
+// full-width input; key indices are checked when the table is built.
 int enqueue_encrypt(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *in, uint32_t *out, size_t n, cudaStream_t st,
-                    const uint32_t *key_idx = nullptr, const uint32_t *groups = nullptr,
-                    uint32_t align = pmk::kGroupAlign) {
-  const uint32_t S = ks->nbits / 32;
-  int rc = pmk::launch_range_check(ks->d_keys, ks->K, S, in, n, ctx->d_status, st, key_idx);
-  if (rc == PMK_OK)
-    rc = pmk::launch_modexp(pmk::ExpMode::kEncrypt, S, call_cfg(ctx, ks, false, n), ks->d_keys, ks->K, in, out, n, st,
-                            ks->nprimes, groups, align);
-  return rc;
+                    const uint32_t *groups = nullptr, uint32_t align = pmk::kGroupAlign) {
+  return pmk::launch_modexp(pmk::ExpMode::kEncrypt, ks->nbits / 32, call_cfg(ctx, ks, false, n), ks->d_keys, ks->K, in,
+                            out, n, st, ks->nprimes, groups, align, ctx->d_status);
 }
 
 // One residue per prime of each chunk (exponent d mod (r_i - 1), or r_i - 2
@@ -249,11 +245,11 @@ int enqueue_decrypt(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *in, uint
                     cudaStream_t st, const uint32_t *key_idx = nullptr, const uint32_t *groups = nullptr,
                     uint32_t align = pmk::kGroupAlign) {
   const uint32_t S = ks->nbits / 32;
-  int rc = pmk::launch_range_check(ks->d_keys, ks->K, S, in, n, ctx->d_status, st, key_idx);
-  if (rc != PMK_OK) return rc;
   if (!use_crt)
     return pmk::launch_modexp(pmk::ExpMode::kDecrypt, S, call_cfg(ctx, ks, false, n), ks->d_keys, ks->K, in, out, n, st,
-                              ks->nprimes, groups, align);
+                              ks->nprimes, groups, align, ctx->d_status);
+  const int rc = pmk::launch_range_check(ks->d_keys, ks->K, S, in, n, ctx->d_status, st, key_idx);
+  if (rc != PMK_OK) return rc;
   return enqueue_crt(ctx, ks, pmk::ExpMode::kCrtHalf, in, out, n, st, nullptr, groups, align);
 }
 
@@ -686,7 +682,7 @@ int pmk_encrypt_chunks(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *d_in,
   const uint32_t *groups = nullptr;
   const uint32_t align = d_key_idx ? group_align(ctx, ks, false, n_chunks) : pmk::kGroupAlign;
   rc = key_groups_for(ctx, ks, d_key_idx, n_chunks, st, align, &groups);
-  if (rc == PMK_OK) rc = enqueue_encrypt(ctx, ks, d_in, d_out, n_chunks, st, d_key_idx, groups, align);
+  if (rc == PMK_OK) rc = enqueue_encrypt(ctx, ks, d_in, d_out, n_chunks, st, groups, align);
   if (d_key_idx) release(ctx->grp, st);
   return rc;
 }

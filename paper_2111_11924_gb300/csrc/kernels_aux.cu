@@ -644,7 +644,7 @@ int launch_modexp_tasks(uint32_t limbs, KernelConfig cfg, bool crt, const BatchT
 
 int launch_modexp(ExpMode mode, uint32_t limbs, KernelConfig cfg, const KeyDev *keys, uint32_t K, const uint32_t *in,
                   uint32_t *out, size_t n, cudaStream_t st, uint32_t parts, const uint32_t *groups,
-                  uint32_t groups_align) {
+                  uint32_t groups_align, uint32_t *status) {
   if (n == 0) return PMK_OK;
   const bool crt = mode == ExpMode::kCrtHalf || mode == ExpMode::kCrtInverse;
   if (crt && (parts < 2 || parts > (uint32_t)kMaxPrimes)) return PMK_EINVAL;
@@ -663,7 +663,8 @@ int launch_modexp(ExpMode mode, uint32_t limbs, KernelConfig cfg, const KeyDev *
   int sel = (mode == ExpMode::kEncrypt || mode == ExpMode::kCrtInverse) ? 1 : 0;
   int np = crt ? (int)parts : 1;
   void *args[] = {(void *)&keys, (void *)&K,   (void *)&in, (void *)&out,
-                  (void *)&nl,   (void *)&sel, (void *)&np, (void *)&groups};
+                  (void *)&nl,   (void *)&sel, (void *)&np, (void *)&groups,
+                  (void *)&status};
   return cuda_rc(cudaLaunchKernel(e->fn, grid, dim3(e->threads), args, e->smem, st));
 }
 

@@ -153,9 +153,10 @@ __device__ __forceinline__ uint32_t resolve(uint32_t (&t)[L], uint32_t c0, uint3
 }
 
 // Subtract N once if the value (topw above t, topw in the top lane) is at
-// least N.  Returns the new word above limb S - 1 (top lane only).
+// least N.  Returns whether it was, and the new word above limb S - 1 in topw
+// (top lane only).
 template <int L, int TPI>
-__device__ __forceinline__ uint32_t reduce_once(uint32_t (&t)[L], uint32_t topw, const uint32_t (&nn)[L], uint32_t r) {
+__device__ __forceinline__ bool reduce_once(uint32_t (&t)[L], uint32_t &topw, const uint32_t (&nn)[L], uint32_t r) {
   const bool top = (r == TPI - 1);
   uint32_t d[L], b;
   sub_cc(d[0], t[0], nn[0]);
@@ -183,14 +184,14 @@ __device__ __forceinline__ uint32_t reduce_once(uint32_t (&t)[L], uint32_t topw,
     for (int j = 0; j < L; j++) t[j] = d[j];
     topw -= b;
   }
-  return topw;
+  return ge;
 }
 
 // Resolve pending words and reduce the value once by N, leaving the canonical
 // result (< N) in t.  Requires the value < 2N.
 template <int L, int TPI>
 __device__ __forceinline__ void finalize(uint32_t (&t)[L], uint32_t c0, const uint32_t (&nn)[L], uint32_t r) {
-  const uint32_t topw = resolve<L, TPI>(t, c0, r);
+  uint32_t topw = resolve<L, TPI>(t, c0, r);
   reduce_once<L, TPI>(t, topw, nn, r);
 }
 
@@ -648,7 +649,7 @@ __device__ __forceinline__ void make_modulus(Modulus<S / TPI> &m, const uint32_t
 #pragma unroll
       for (int j = 1; j < L; j++) addc_cc(m.f[j], m.f[j], j == L - 1 ? n2 : j == L - 2 ? n1 : m.n[j]);
       addc(g, 0u, 0u);
-      const uint32_t topw = resolve<L, TPI>(m.f, g, r);
+      uint32_t topw = resolve<L, TPI>(m.f, g, r);
       reduce_once<L, TPI>(m.f, topw, m.n, r);
     }
     uint32_t t1 = m.n[L - 1], t0 = m.n[L - 2];
@@ -718,7 +719,7 @@ __device__ __forceinline__ void mont_mul_pairs(uint32_t (&a)[S / TPI], const uin
   t.reduce(m);
   const uint32_t pending = t.shift_out(a);
   uint32_t topw = resolve<L, TPI>(a, pending, r);
-  topw = reduce_once<L, TPI>(a, topw, m.n, r);
+  reduce_once<L, TPI>(a, topw, m.n, r);
   if (m.tight) reduce_once<L, TPI>(a, topw, m.n, r);
 }
 

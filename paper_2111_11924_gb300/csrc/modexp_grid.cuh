@@ -89,11 +89,13 @@ __device__ __forceinline__ long long slot_chunk(const uint32_t *__restrict__ grp
 // instances in an SM's shared memory).  TABLE (kTableFull or kTableSmall)
 // sizes the odd-power tables in shared memory and selects the key's
 // schedules built for it.  grp: a key group table (explicit key indices), or
-// null for round robin.
+// null for round robin.  With `status`, a full-width input not below its
+// modulus sets kStatusRange.
 template <int S, int TPI, bool CRT, int NT = kThreads, int TABLE = kTableFull>
 __global__ void __launch_bounds__(NT, 1) k_modexp(const KeyDev *__restrict__ keys, uint32_t K,
                                                const uint32_t *__restrict__ in, uint32_t *__restrict__ out,
-                                               long long n, int sel, int parts, const uint32_t *__restrict__ grp) {
+                                               long long n, int sel, int parts, const uint32_t *__restrict__ grp,
+                                               uint32_t *__restrict__ status) {
   constexpr int L = S / TPI;
   constexpr int IPB = NT / TPI;
   constexpr int ROW = Layout<S>::kRow;
@@ -144,12 +146,25 @@ __global__ void __launch_bounds__(NT, 1) k_modexp(const KeyDev *__restrict__ key
     }
     // Encryption takes x as it is: its exponent walk gives x^e R^-(e-1), and
     // the last product with R^e mod N the result, one product of 19 less
-    // (encrypting 100 MiB at 2048 bits: 7.43 and 6.97 ms).  As an operand x has to be below N.
+    // (encrypting 100 MiB at 2048 bits: 7.43 and 6.97 ms).
+    // Encryption takes x mod N as it is: its exponent walk gives x^e R^-(e-1),
+    // and the last product with R^e mod N the result, one product of 19 less
+    // (encrypting 100 MiB at 2048 bits: 7.43 and 6.97 ms).  The range is
+    // checked here and not by a launch of its own (encrypting 1 KiB: 34.3 and
+    // 30.8 us a call); decryption checks a copy, since checking x itself
+    // changed how ptxas schedules the 64-limb, 16-lane products (3% slower).
+    uint32_t top = 0;
+    bool over;
     if (sel) {
-      reduce_once<L, TPI>(a, 0u, m.n, r);
+      over = reduce_once<L, TPI>(a, top, m.n, r);
     } else {
+      uint32_t c[L];
+#pragma unroll
+      for (int j = 0; j < L; j++) c[j] = a[j];
+      over = reduce_once<L, TPI>(c, top, m.n, r);
       mont<S, TPI>(a, sR2, m, r);  // x R mod N
     }
+    if (over && status && r == 0) report(status, kStatusRange, t);
   } else {
     crt_input<S, TPI>(a, in + t * W, active, parts, sR2, sR3, m, r);
   }

@@ -66,7 +66,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_modexp_tasks(const BatchTask *_
         for (int j = 0; j < L; j++) a[j] = 0;
       }
       if (enc) {
-        reduce_once<L, TPI>(a, 0u, m.n, r);
+        uint32_t top = 0;
+        reduce_once<L, TPI>(a, top, m.n, r);
       } else {
         mont<S, TPI>(a, sR2, m, r);
       }

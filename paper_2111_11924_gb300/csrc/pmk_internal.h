@@ -199,10 +199,12 @@ uint32_t crt_sum_block_instances(uint32_t limbs);
 // CRT modes run `parts` residues per chunk (the key's prime count) over
 // `limbs` = s / parts limbs each; residue i of chunk t goes to out[t][i * limbs].
 // With `groups` (a table of launch_key_groups built with alignment
-// groups_align) chunks are taken by key group instead of round robin.
+// groups_align) chunks are taken by key group instead of round robin.  With
+// `status`, the full-width modes flag chunks >= their key's modulus
+// (kStatusRange), as launch_range_check does.
 int launch_modexp(ExpMode mode, uint32_t limbs, KernelConfig cfg, const KeyDev *keys, uint32_t K, const uint32_t *in,
                   uint32_t *out, size_t n, cudaStream_t st, uint32_t parts = 2, const uint32_t *groups = nullptr,
-                  uint32_t groups_align = kGroupAlign);
+                  uint32_t groups_align = kGroupAlign, uint32_t *status = nullptr);
 // CRT recombination of `parts` residues per chunk (limbs / parts limbs
 // each) in place at full width `limbs`: out[t] holds the residues and
 // receives the value mod N.
