@@ -284,6 +284,61 @@ int key_groups_for(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *key_idx, 
   return rc;
 }
 
+// A *_host call in pieces: each piece's copy in, kernels and copy out are
+// queued on one of kPieceStreams streams, so that the copies of one piece run
+// beside the kernels of the others and a piece's last blocks beside the next
+// one's first.  A piece is at least kPieceBytes of message, enough to fill the
+// GPU several times, and starts at a multiple of K chunks (chunk t of the
+// message is chunk t - start of the piece under the same key) and of 16
+// (aligned message bytes).  Measured, one piece on one stream against pieces:
+// encrypting 100 MiB at 2048 bits 8.04 and 7.14 ms, 50 MB at 1024 bits 2.29
+// and 1.90; CRT decryption of 25 MB 58.5 and 58.3.
+constexpr size_t kPieceBytes = 6u << 20, kMaxPieces = 8;
+
+// Chunks per piece for a message of n chunks (n itself: one piece).
+size_t piece_chunks(size_t msg_len, size_t n, uint32_t K) {
+  const size_t pieces = std::min(kMaxPieces, msg_len / kPieceBytes);
+  if (pieces < 2) return n;
+  size_t unit = K;
+  while (unit % 16) unit *= 2;
+  return std::min(n, ((n + pieces - 1) / pieces + unit - 1) / unit * unit);
+}
+
+// queue(first chunk, chunks, stream) for every piece.  With one piece that is
+// the caller's stream; else `st` has everything queued before the pieces begin
+// and waits for them all.  On an error the piece streams are idle on return.
+template <typename Queue>
+int in_pieces(pmk_ctx *ctx, size_t msg_len, size_t n, uint32_t K, cudaStream_t st, Queue queue) {
+  const size_t per = piece_chunks(msg_len, n, K);
+  if (per == n) return queue((size_t)0, n, st);
+  pmk::PieceStreams &p = ctx->pieces;
+  if (!p.start && cudaEventCreateWithFlags(&p.start, cudaEventDisableTiming) != cudaSuccess) return PMK_ECUDA;
+  for (int i = 0; i < pmk::kPieceStreams; i++)
+    if ((!p.s[i] && cudaStreamCreateWithFlags(&p.s[i], cudaStreamNonBlocking) != cudaSuccess) ||
+        (!p.done[i] && cudaEventCreateWithFlags(&p.done[i], cudaEventDisableTiming) != cudaSuccess))
+      return PMK_ECUDA;
+  int rc = cudaEventRecord(p.start, st) == cudaSuccess ? PMK_OK : PMK_ECUDA;
+  for (int i = 0; i < pmk::kPieceStreams && rc == PMK_OK; i++)
+    if (cudaStreamWaitEvent(p.s[i], p.start, 0) != cudaSuccess) rc = PMK_ECUDA;
+  for (size_t first = 0, i = 0; first < n && rc == PMK_OK; first += per, i++)
+    rc = queue(first, std::min(per, n - first), p.s[i % pmk::kPieceStreams]);
+  for (int i = 0; i < pmk::kPieceStreams && rc == PMK_OK; i++)
+    if (cudaEventRecord(p.done[i], p.s[i]) != cudaSuccess || cudaStreamWaitEvent(st, p.done[i], 0) != cudaSuccess)
+      rc = PMK_ECUDA;
+  if (rc != PMK_OK)
+    for (cudaStream_t x : p.s) cudaStreamSynchronize(x);
+  return rc;
+}
+
+void drop(pmk::PieceStreams &p) {
+  for (cudaStream_t x : p.s)
+    if (x) cudaStreamDestroy(x);
+  for (cudaEvent_t e : p.done)
+    if (e) cudaEventDestroy(e);
+  if (p.start) cudaEventDestroy(p.start);
+  p = pmk::PieceStreams{};
+}
+
 }  // namespace
 
 namespace pmk {
@@ -328,6 +383,7 @@ void pmk_destroy(pmk_ctx *ctx) {
   drop(ctx->a);
   drop(ctx->b);
   drop(ctx->grp);
+  drop(ctx->pieces);
   cudaFree(ctx->d_status);
   delete ctx;
 }
@@ -815,22 +871,26 @@ int pmk_encrypt_message_host(pmk_ctx *ctx, const pmk_keyset *ks, const uint8_t *
   if (!h_msg || !h_cipher) return PMK_EINVAL;
   DeviceGuard g(ctx->device);
   if (!g.ok()) return PMK_ECUDA;
-  const size_t words = n_chunks * (ks->nbits / 32);
+  const size_t S = ks->nbits / 32, P = pmk_payload_bytes(ks->nbits);
   cudaStream_t st = as_stream(stream);
   int rc = acquire(ctx->msg, msg_len, st);
-  if (rc == PMK_OK) rc = acquire(ctx->a, words * 4, st);
+  if (rc == PMK_OK) rc = acquire(ctx->a, n_chunks * S * 4, st);
   uint8_t *m = static_cast<uint8_t *>(ctx->msg.ptr);
   uint32_t *c = static_cast<uint32_t *>(ctx->a.ptr);
   bool queued = false;  // a copy from or to the caller's host memory is in flight
-  if (rc == PMK_OK) {
-    queued = true;
-    if (cudaMemcpyAsync(m, h_msg, msg_len, cudaMemcpyHostToDevice, st) != cudaSuccess) rc = PMK_ECUDA;
-  }
-  if (rc == PMK_OK && pmk::fault_injected("after_copy")) rc = PMK_ECUDA;
-  if (rc == PMK_OK) rc = pmk::launch_split(ks->nbits, m, msg_len, c, n_chunks, st);
-  if (rc == PMK_OK) rc = enqueue_encrypt(ctx, ks, c, c, n_chunks, st);
-  if (rc == PMK_OK && cudaMemcpyAsync(h_cipher, c, words * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-    rc = PMK_ECUDA;
+  if (rc == PMK_OK)
+    rc = in_pieces(ctx, msg_len, n_chunks, ks->K, st, [&](size_t first, size_t n, cudaStream_t s) -> int {
+      const size_t byte0 = first * P, len = std::min(n * P, msg_len - byte0);
+      uint32_t *cp = c + first * S;
+      queued = true;
+      if (cudaMemcpyAsync(m + byte0, h_msg + byte0, len, cudaMemcpyHostToDevice, s) != cudaSuccess) return PMK_ECUDA;
+      if (pmk::fault_injected("after_copy")) return PMK_ECUDA;
+      int r = pmk::launch_split(ks->nbits, m + byte0, len, cp, n, s);
+      if (r == PMK_OK) r = enqueue_encrypt(ctx, ks, cp, cp, n, s);
+      if (r == PMK_OK && cudaMemcpyAsync(h_cipher + first * S, cp, n * S * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+        r = PMK_ECUDA;
+      return r;
+    });
   release(ctx->msg, st);
   release(ctx->a, st);
   if (rc != PMK_OK) {
@@ -849,7 +909,7 @@ int pmk_decrypt_message_host(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t 
   if (!h_msg || !h_cipher) return PMK_EINVAL;
   DeviceGuard g(ctx->device);
   if (!g.ok()) return PMK_ECUDA;
-  const size_t words = n_chunks * (ks->nbits / 32);
+  const size_t S = ks->nbits / 32, P = pmk_payload_bytes(ks->nbits), words = n_chunks * S;
   cudaStream_t st = as_stream(stream);
   int rc = acquire(ctx->msg, msg_len, st);
   if (rc == PMK_OK) rc = acquire(ctx->a, words * 4, st);
@@ -857,14 +917,18 @@ int pmk_decrypt_message_host(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t 
   uint8_t *m = static_cast<uint8_t *>(ctx->msg.ptr);
   uint32_t *c = static_cast<uint32_t *>(ctx->a.ptr), *p = static_cast<uint32_t *>(ctx->b.ptr);
   bool queued = false;  // a copy from or to the caller's host memory is in flight
-  if (rc == PMK_OK) {
-    queued = true;
-    if (cudaMemcpyAsync(c, h_cipher, words * 4, cudaMemcpyHostToDevice, st) != cudaSuccess) rc = PMK_ECUDA;
-  }
-  if (rc == PMK_OK && pmk::fault_injected("after_copy")) rc = PMK_ECUDA;
-  if (rc == PMK_OK) rc = enqueue_decrypt(ctx, ks, c, p, n_chunks, use_crt, st);
-  if (rc == PMK_OK) rc = pmk::launch_join(ks->nbits, p, n_chunks, m, msg_len, st);
-  if (rc == PMK_OK && cudaMemcpyAsync(h_msg, m, msg_len, cudaMemcpyDeviceToHost, st) != cudaSuccess) rc = PMK_ECUDA;
+  if (rc == PMK_OK)
+    rc = in_pieces(ctx, msg_len, n_chunks, ks->K, st, [&](size_t first, size_t n, cudaStream_t s) -> int {
+      const size_t byte0 = first * P, len = std::min(n * P, msg_len - byte0), w = first * S;
+      queued = true;
+      if (cudaMemcpyAsync(c + w, h_cipher + w, n * S * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) return PMK_ECUDA;
+      if (pmk::fault_injected("after_copy")) return PMK_ECUDA;
+      int r = enqueue_decrypt(ctx, ks, c + w, p + w, n, use_crt, s);
+      if (r == PMK_OK) r = pmk::launch_join(ks->nbits, p + w, n, m + byte0, len, s);
+      if (r == PMK_OK && cudaMemcpyAsync(h_msg + byte0, m + byte0, len, cudaMemcpyDeviceToHost, s) != cudaSuccess)
+        r = PMK_ECUDA;
+      return r;
+    });
   release(ctx->msg, st);
   release(ctx->a, st);
   release(ctx->b, st);

@@ -285,6 +285,16 @@ namespace pmk {
 constexpr size_t kDirectMaxJobs = 256;
 }  // namespace pmk
 
+namespace pmk {
+// The streams over which a *_host call spreads the pieces of a long message
+// (made on first use; idle between calls).
+constexpr int kPieceStreams = 3;
+struct PieceStreams {
+  cudaStream_t s[kPieceStreams] = {};
+  cudaEvent_t start = nullptr, done[kPieceStreams] = {};
+};
+}  // namespace pmk
+
 // Context: one device, its status record, staging and kernel geometry choices.
 struct pmk_ctx {
   int device = 0;
@@ -292,6 +302,7 @@ struct pmk_ctx {
   uint32_t *d_status = nullptr;            // status record: error bits, smallest failing chunk
   pmk::Staging msg, a, b;                  // staging of the *_host calls and the blinded CRT path
   pmk::Staging grp;                        // key-group table of calls with explicit key indices
+  pmk::PieceStreams pieces;
   std::map<uint32_t, pmk::KernelConfig> cfg;  // (limbs << 1 | crt) -> kernel geometry override
   std::map<uint32_t, int> table;              // (limbs << 1 | crt) -> odd-power table size override
   size_t batch_direct_max = pmk::kDirectMaxJobs;  // pmk_set_batch_direct_max
