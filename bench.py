@@ -45,18 +45,18 @@ WORKLOAD = W.FILE_1MIB_2048
 METRIC = "2048-bit decrypt chunk-modexps/s"
 UNIT = "chunk-modexps/s"
 L2_FLUSH_BYTES = 256 << 20
-FORM_NAMES = ["chain", "columns"]  # Montgomery product forms (pmk_set_kernel_config)
-KERNELS_PER_STEP = 6  # split, range check + modexp (encrypt), range check + modexp (decrypt), join
+FORM_NAMES = ["pairs", "pairs"]  # the product behind both values of pmk_set_kernel_config's form
+KERNELS_PER_STEP = 4  # split, modexp (encrypt), modexp (decrypt), join
 
 # ncu counters of the full-d decryption kernel on the 1 MiB workload, valid
 # only for the kernel sources they were measured on (see profiles/): DRAM
 # bytes per launch, and the issue-slot and pipe utilisation that the
-# algorithmic count does not see (carry adds and column shifts take issue
-# slots of their own).
+# algorithmic count does not see (chain ends and shifts take issue slots of
+# their own).
 TRAFFIC_SOURCES = ["paper_2111_11924_gb300/csrc/modexp_core.cuh", "paper_2111_11924_gb300/csrc/modexp_grid.cuh"]
 COUNTERS_MEASURED = {  # source digest -> counters of one launch
-    "5829c9343745b4f4": {"traffic": 1273600, "issue_active_pct": 50.80, "warps_active_per_sm": 6.93,
-                         "alu_pipe_pct": 57.17, "fmaheavy_pipe_pct": 60.34, "warp_instructions": 10037561520},
+    "c6b9175443a88cc2": {"traffic": 1150208, "issue_active_pct": 32.88, "warps_active_per_sm": 6.99,
+                         "alu_pipe_pct": 18.94, "fmaheavy_pipe_pct": 77.79, "warp_instructions": 4223030943},
 }
 
 
@@ -449,7 +449,7 @@ def run_ours(args):
                      "frac": achieved / peak_tops, "traffic": counters.get("traffic"),
                      "issue_slots": issue_slots(counters, alg_macs),
                      "kernel": f"k_modexp<64,{tuned['tpi']},full,{FORM_NAMES[tuned['form']]}> "
-                               "(full-d decrypt; interval includes its ~4 us range check)",
+                               "(full-d decrypt, its range check included)",
                      "ops_per_launch": 2 * alg_macs, "ops_basis": "2 INT32 multiply-add halves per 32x32->64 MAC; "
                      f"{algorithmic_montmuls(w.nbits):.1f} Montgomery products x {macs_per_montmul(w.nbits)} MACs "
                      f"x {n} chunks", "decrypt_ms": dec_ms,

@@ -22,9 +22,10 @@ BlindEntry make_blind() {
 // those with more lanes per instance.
 const BlindEntry *blind_entries(int *count) {
   static const BlindEntry entries[] = {
-      make_blind<2, 2>(),   make_blind<4, 2>(),   make_blind<8, 2>(),   make_blind<16, 2>(),  make_blind<16, 8, 32>(),
-      make_blind<32, 4, 64>(), make_blind<32, 8, 32>(), make_blind<32, 16, 32>(), make_blind<48, 8>(), make_blind<48, 16, 32>(),
-      make_blind<64, 8>(),  make_blind<64, 16, 32>(), make_blind<64, 32, 32>(), make_blind<96, 8>(),  make_blind<96, 16, 32>(),
+      make_blind<2, 2>(), make_blind<4, 2>(), make_blind<8, 2>(), make_blind<16, 2>(),
+      make_blind<16, 8, 32>(), make_blind<32, 4, 64>(), make_blind<32, 8, 32>(), make_blind<32, 16, 32>(),
+      make_blind<48, 8>(), make_blind<48, 16, 32>(), make_blind<64, 8>(), make_blind<64, 16, 32>(),
+      make_blind<64, 32, 32>(), make_blind<96, 8>(), make_blind<96, 16, 32>(), make_blind<96, 32, 32>(),
       make_blind<128, 16>(), make_blind<128, 32, 32>(),
   };
   *count = (int)(sizeof(entries) / sizeof(entries[0]));

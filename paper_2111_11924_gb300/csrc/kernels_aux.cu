@@ -555,10 +555,9 @@ long long product_clocks(int limbs, int tpi, const Load &load, int sms) {
 
 // More lanes shorten one exponentiation and cost more in total, so they pay
 // while the GPU has schedulers to spare.  Measured, ms by lanes: full d at
-// 2048 bits, 403 chunks 8.06 (8 lanes) / 4.55 (16) / 3.09 (32), 1,024 chunks
-// 8.07 / 4.56 / 4.46, 2,056 chunks 8.07 / 6.61 / 8.18, 4,113 chunks 11.7 / 12.7
-// / 13.9; CRT at 3072 bits, 685 chunks 3.70 (8) / 3.41 (16), 6,000 chunks 12.7
-// / 14.9.  Fewer lanes than the default are not considered: their tables
+// 2048 bits, 403 chunks 7.95 (8 lanes) / 4.43 (16) / 2.95 (32), 2,056 chunks
+// 7.95 / 6.38 / 7.77, 4,113 chunks 11.4 / 12.3 / 13.1; CRT at 3072 bits, 685
+// chunks 3.66 (8) / 3.31 (16), 6,000 chunks 12.6 / 14.7.  Fewer lanes than the default are not considered: their tables
 // leave too few exponentiations on an SM.
 KernelConfig config_for_load(uint32_t limbs, bool crt, const Load &load, int sms) {
   KernelConfig best = default_config(limbs, crt);

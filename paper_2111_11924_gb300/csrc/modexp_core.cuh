@@ -3,11 +3,11 @@
 // One exponentiation ("instance") is held by TPI consecutive lanes of a warp;
 // lane r keeps limbs [r L, r L + L) of every S-limb value in registers
 // (L = S / TPI).  The multiplication is Algorithm 3 (Montgomery) in its
-// word-serial CIOS form (Koc, Acar, Kaliski 1996) with r = 2^32 per row and
-// R = 2^(32 S) overall:
-//     for i in 0..S-1:  T += a * y_i;  q = T_0 * n0 mod 2^32;  T += q N;  T /= 2^32
-// followed by one conditional subtraction, so every product is canonical
-// (< N).  Exponentiation is Algorithm 2's square-and-multiply generalised to a
+// word-serial CIOS form (Koc, Acar, Kaliski 1996), R = 2^(32 S), two words of
+// the multiplier a step:
+//     for i in 0, 2, .. S-2:  T += a (y_i + 2^32 y_{i+1});  T = (T + q N) / 2^64
+// with q so that T + q N is divisible (how q is found: PairSum), followed by
+// one conditional subtraction, so every product is canonical (< N).  Exponentiation is Algorithm 2's square-and-multiply generalised to a
 // left-to-right sliding window of odd powers (schedules built on the host).
 //
 // Cost model on this GPU (measured with row-shaped loops, MAC per clock per SM
@@ -17,7 +17,10 @@
 // 63 / 64.  The multiplier's high half bounds every form, and the adds are
 // free only inside the multiply-add, so a row is built of carry chains over
 // 64-bit pairs: one instruction per MAC and nothing but the chain ends on the
-// ALU pipe.
+// ALU pipe.  (Forming each cross product of a squaring once was built on top
+// of this and left out: 804 instead of 1,024 multiply-adds a lane at 64 limbs
+// on 8 lanes, but 400 more adds and moves; the same speed with two warps per
+// scheduler, 4% faster with three, and 6% slower at 32 limbs on 4 lanes.)
 // Lane-to-lane carries are deferred: a lane keeps small pending words above
 // its L limbs; after the last row a ballot carry-lookahead resolves them in
 // O(1) warp operations.
@@ -250,8 +253,8 @@ __host__ __device__ constexpr bool ring() {
 
 // A modulus N as the products use it: this lane's limbs of N, and for two or
 // more limbs per lane (see PairSum) of f = F, or F - 2^(32 (S - 2)) mod N with
-// ring(), where F = (k N + 1) / 2^64 and k = -N^-1 mod 2^64.  tight: N is so near 2^(32 S) that a product can reach
-// 2N before its last subtraction.
+// ring(), where F = (k N + 1) / 2^64 and k = -N^-1 mod 2^64.  tight: N is so
+// near 2^(32 S) that a product can reach 2N before its last subtraction.
 template <int L>
 struct Modulus {
   uint32_t n[L], f[L];
@@ -260,7 +263,7 @@ struct Modulus {
 };
 
 // a <- MontMul(a, y) = a y R^-1 mod N.  a: this lane's limbs (any value < R);
-// ys: y's S limbs in shared memory (y < N), read as 16-byte broadcasts.
+// ys: y's S limbs in shared or global memory (y < N).
 // One row at a time, one add-with-carry chain per lane: the form for one limb
 // per lane (the residues of 128-bit keys), which has no pairs.
 template <int S, int TPI>
@@ -370,7 +373,6 @@ struct PairSum {
   uint32_t e[L + 2], o[L], c2;  // c2: weight 2^(32 (L + 2))
   uint32_t x0, x1, q0, q1;      // from the lane above (its words 0, 1), and the quotient
   int above;                    // the lane above; lane 0 for the top lane
-
   uint32_t keep;                // zero in the top lane, unless ring()
 
   __device__ __forceinline__ explicit PairSum(uint32_t r)
@@ -501,7 +503,6 @@ struct OddPairSum {
   uint32_t e[L + 1], o[L + 1], c1, c2;  // c1, c2: weights 2^(32 (L + 1)), 2^(32 (L + 2))
   uint32_t x0, x1, q0, q1;
   int above;
-
   uint32_t keep;                // zero in the top lane, unless ring()
 
   __device__ __forceinline__ explicit OddPairSum(uint32_t r)
@@ -681,11 +682,13 @@ __host__ __device__ constexpr int unrolled_steps() {
 // a: any value < R; ys: y's S limbs in shared or global memory (y < N).
 //
 // Bound: the wide multiply-add, 4 L per lane and step at 4 clocks of the
-// fma-heavy pipe each, against about 20 other instructions a step; a single
-// warp issues one per 6.6 clocks, two nearly fill the pipe.  Measured (2048-bit
-// keys, full d, default geometry): 1 MiB
-// 17.63 ms with 64-bit columns, 12.66 with two-row steps and a quotient by
-// product, 11.68 now; 10 MiB 142.3, 104.1, 94.6; CRT 1 MiB 4.63, 3.34, 3.10.
+// fma-heavy pipe each, against about 20 other instructions a step (64 limbs
+// on 8 lanes: 1,028 instructions on that pipe and 680 others a product).  A
+// single warp issues one per 6.6 clocks; two warps per scheduler take 9,700
+// clocks for a product each, 85% of the pipe, three or more 4,650 per product.
+// Measured, 2048-bit keys, default geometry, in ms with 64-bit columns / pairs
+// and a quotient by product / now: full d 1 MiB 17.63 / 12.66 / 11.40, 10 MiB
+// 142.3 / 104.1 / 93.1; CRT 1 MiB 4.63 / 3.34 / 3.08.
 template <int S, int TPI, bool HOT>
 __device__ __forceinline__ void mont_mul_pairs(uint32_t (&a)[S / TPI], const uint32_t *ys, const Modulus<S / TPI> &m,
                                                uint32_t r) {
@@ -746,11 +749,10 @@ __device__ __forceinline__ void mod_add(uint32_t (&a)[L], const uint32_t (&b)[L]
 }
 
 // Table of odd powers and the exponent walk.  On entry a = x in Montgomery
-// form; on exit a = MontMul(x^E in Montgomery form, last) (of any x < N:
-// x^E R^-E last mod N).  tbl: the instance's odd-power
-// table (at least maxidx + 1 rows: the table size the schedule was built
-// for), ybuf: one row of this instance.  sched: steps of make_schedule()
-// (block-uniform).  Squarings and multiplications share one product in the
+// form; on exit a = MontMul(x^E in Montgomery form, last), that is, for any
+// x < N, x^E R^-E last mod N.  tbl: the instance's odd-power table (at least
+// maxidx + 1 rows: the table size the schedule was built for), ybuf: one row
+// of this instance.  sched: steps of make_schedule() (warp-uniform).  Squarings and multiplications share one product in the
 // code, so that it can be unrolled whole.
 template <int S, int TPI>
 __device__ __forceinline__ void exp_window(uint32_t (&a)[S / TPI], uint32_t *tbl, uint32_t *ybuf,

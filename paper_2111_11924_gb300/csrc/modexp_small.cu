@@ -1,10 +1,11 @@
 // CRT residue kernels with the small odd-power table (8 odd powers, windows
 // up to 4 bits): half the shared memory per exponentiation, so more are
 // resident per SM, for a few percent more products.  Measured on GB300 it
-// pays only where the residues fill the GPU many times over (2048-bit CRT
-// on 100 MiB); the autotuner decides per key set and batch size.  The
-// full-width kernels measured slower with it at every size and are not built
-// with it.
+// pays for 16 limbs on 2 lanes only (1024-bit CRT, 33,000 chunks 2.94 and
+// 2.84 ms; at 32 limbs on 4 lanes 24.73 and 24.84 ms on 41,121 chunks, and
+// 1-2.5% slower elsewhere); the autotuner decides per key set and batch size.
+// The full-width kernels measured slower with it at every size and are not
+// built with it.
 #include "modexp_kernels.cuh"
 
 namespace pmk {
