@@ -312,10 +312,10 @@ int pmk_decrypt_message_host(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t 
  *   whose GPU work overlaps (other streams, other host threads) race and
  *   corrupt each other's results.
  *   The call ends by synchronising `stream`, so it must not be made while
- *   `stream` is being captured into a CUDA graph.  It runs the built-in
- *   default kernel geometry and odd-power table of each width, not a
- *   context's autotuned ones (it takes no context), so its speed can differ
- *   from pmk_decrypt_message_host's.
+ *   `stream` is being captured into a CUDA graph.  It runs the kernel
+ *   geometry that the library chooses for the call's size and the default
+ *   odd-power table, not a context's autotuned ones (it takes no context),
+ *   so its speed can differ from pmk_decrypt_message_host's.
  *   Returns PMK_OK, PMK_ERANGE (a chunk >= its modulus), PMK_EINVAL (NULL
  *   key set or buffer, a chunk count that does not match msg_len, or 2^32
  *   chunks or more), PMK_ETOOLARGE or PMK_ECUDA.  On an error after the copy
