@@ -288,29 +288,35 @@ int key_groups_for(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *key_idx, 
 // queued on one of kPieceStreams streams, so that the copies of one piece run
 // beside the kernels of the others and a piece's last blocks beside the next
 // one's first.  A piece is at least kPieceBytes of message, enough to fill the
-// GPU several times, and starts at a multiple of K chunks (chunk t of the
-// message is chunk t - start of the piece under the same key) and of 16
-// (aligned message bytes).  Measured, one piece on one stream against pieces:
+// GPU several times, has kPieceRows chunks a key at least (a block serves one
+// key: the last block of each is part empty), and starts at a multiple of K
+// chunks (chunk t of the message is chunk t - start of the piece under the
+// same key) and of 16 (aligned message bytes).  Host buffers that overlap go
+// in one piece (all input is read before any output is written), and so does
+// a call on a stream of another priority than the pieces' own.  Measured, one piece on one stream against pieces:
 // encrypting 100 MiB at 2048 bits 8.04 and 7.14 ms, 50 MB at 1024 bits 2.29
 // and 1.90; CRT decryption of 25 MB 58.5 and 58.3.
-constexpr size_t kPieceBytes = 6u << 20, kMaxPieces = 8;
+constexpr size_t kPieceBytes = 6u << 20, kPieceRows = 128, kMaxPieces = 8;
 
 // Chunks per piece for a message of n chunks (n itself: one piece).
 size_t piece_chunks(size_t msg_len, size_t n, uint32_t K) {
-  const size_t pieces = std::min(kMaxPieces, msg_len / kPieceBytes);
+  const size_t pieces = std::min({kMaxPieces, msg_len / kPieceBytes, n / (kPieceRows * K)});
   if (pieces < 2) return n;
   size_t unit = K;
   while (unit % 16) unit *= 2;
   return std::min(n, ((n + pieces - 1) / pieces + unit - 1) / unit * unit);
 }
 
-// queue(first chunk, chunks, stream) for every piece.  With one piece that is
-// the caller's stream; else `st` has everything queued before the pieces begin
-// and waits for them all.  On an error the piece streams are idle on return.
+// queue(first chunk, chunks, stream) for every piece; `split` false asks for
+// one piece.  With one piece that is the caller's stream; else the pieces begin
+// after all that `st` holds, and `st` waits for them all.  On an error the
+// piece streams are idle on return.
 template <typename Queue>
-int in_pieces(pmk_ctx *ctx, size_t msg_len, size_t n, uint32_t K, cudaStream_t st, Queue queue) {
-  const size_t per = piece_chunks(msg_len, n, K);
-  if (per == n) return queue((size_t)0, n, st);
+int in_pieces(pmk_ctx *ctx, bool split, size_t msg_len, size_t n, uint32_t K, cudaStream_t st, Queue queue) {
+  const size_t per = split ? piece_chunks(msg_len, n, K) : n;
+  int priority = 0;  // the piece streams' own
+  if (per < n && cudaStreamGetPriority(st, &priority) != cudaSuccess) return PMK_ECUDA;
+  if (per == n || priority != 0) return queue((size_t)0, n, st);
   pmk::PieceStreams &p = ctx->pieces;
   if (!p.start && cudaEventCreateWithFlags(&p.start, cudaEventDisableTiming) != cudaSuccess) return PMK_ECUDA;
   for (int i = 0; i < pmk::kPieceStreams; i++)
@@ -877,9 +883,10 @@ int pmk_encrypt_message_host(pmk_ctx *ctx, const pmk_keyset *ks, const uint8_t *
   if (rc == PMK_OK) rc = acquire(ctx->a, n_chunks * S * 4, st);
   uint8_t *m = static_cast<uint8_t *>(ctx->msg.ptr);
   uint32_t *c = static_cast<uint32_t *>(ctx->a.ptr);
+  const bool split = !overlap(h_msg, msg_len, h_cipher, n_chunks * S * 4);
   bool queued = false;  // a copy from or to the caller's host memory is in flight
   if (rc == PMK_OK)
-    rc = in_pieces(ctx, msg_len, n_chunks, ks->K, st, [&](size_t first, size_t n, cudaStream_t s) -> int {
+    rc = in_pieces(ctx, split, msg_len, n_chunks, ks->K, st, [&](size_t first, size_t n, cudaStream_t s) -> int {
       const size_t byte0 = first * P, len = std::min(n * P, msg_len - byte0);
       uint32_t *cp = c + first * S;
       queued = true;
@@ -916,9 +923,10 @@ int pmk_decrypt_message_host(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t 
   if (rc == PMK_OK) rc = acquire(ctx->b, words * 4, st);
   uint8_t *m = static_cast<uint8_t *>(ctx->msg.ptr);
   uint32_t *c = static_cast<uint32_t *>(ctx->a.ptr), *p = static_cast<uint32_t *>(ctx->b.ptr);
+  const bool split = !overlap(h_msg, msg_len, h_cipher, n_chunks * S * 4);
   bool queued = false;  // a copy from or to the caller's host memory is in flight
   if (rc == PMK_OK)
-    rc = in_pieces(ctx, msg_len, n_chunks, ks->K, st, [&](size_t first, size_t n, cudaStream_t s) -> int {
+    rc = in_pieces(ctx, split, msg_len, n_chunks, ks->K, st, [&](size_t first, size_t n, cudaStream_t s) -> int {
       const size_t byte0 = first * P, len = std::min(n * P, msg_len - byte0), w = first * S;
       queued = true;
       if (cudaMemcpyAsync(c + w, h_cipher + w, n * S * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) return PMK_ECUDA;

@@ -144,9 +144,6 @@ __global__ void __launch_bounds__(NT, 1) k_modexp(const KeyDev *__restrict__ key
 #pragma unroll
       for (int j = 0; j < L; j++) a[j] = 0;
     }
-    // Encryption takes x as it is: its exponent walk gives x^e R^-(e-1), and
-    // the last product with R^e mod N the result, one product of 19 less
-    // (encrypting 100 MiB at 2048 bits: 7.43 and 6.97 ms).
     // Encryption takes x mod N as it is: its exponent walk gives x^e R^-(e-1),
     // and the last product with R^e mod N the result, one product of 19 less
     // (encrypting 100 MiB at 2048 bits: 7.43 and 6.97 ms).  The range is

@@ -1,10 +1,10 @@
 // Autotuner: for one key set and batch size, time every compiled kernel
-// geometry (lanes per instance) of the exponentiation that the caller will run, with the full odd-power table (window bound 5) and,
-// where compiled, the small one (bound 4), and keep the fastest in the
-// context.  The window
-// width within the bound is chosen per exponent on the host (fewest
-// products); the table size trades a few more products for more resident
-// instances, which only a measurement can settle.
+// geometry (lanes per instance) of the exponentiation that the caller will
+// run, with the full odd-power table (window bound 5) and, where compiled, the
+// small one (bound 4), and keep the fastest in the context.  The window width
+// within the bound is chosen per exponent on the host (fewest products); the
+// table size trades a few more products for more resident instances, which
+// only a measurement can settle.
 //
 // Inputs are synthetic chunks below every modulus (top limb zero), so the
 // timing covers the same schedule lengths as real ciphertexts; results of

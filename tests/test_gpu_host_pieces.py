@@ -38,6 +38,53 @@ def test_pieces_equal_the_device_calls(nbits, K, size):
     ctx.close()
 
 
+def test_overlapping_host_buffers_read_all_input_first():
+    # The output begins half way through the input: written piece by piece it would reach input not yet read.
+    import torch
+
+    import paper_2111_11924_gb300 as P
+
+    nbits, size = 1024, 48 << 20
+    ctx = P.Context(0)
+    ks = ctx.keygen(3, nbits, 65537, 33)
+    msg = torch.from_numpy(np.random.default_rng(2).integers(0, 256, size, dtype=np.uint8))
+    n = P.num_chunks(size, nbits)
+    total = n * nbits // 8
+    want = ctx.encrypt_chunks(ks, ctx.split(nbits, msg.cuda())).cpu()
+    buf = _pinned(2 * total, torch.uint8)
+    buf[:size] = msg
+    off = size // 2 // 16 * 16
+    cipher = buf[off:off + total].view(torch.int32).view(n, nbits // 32)
+    ctx.encrypt_message_host(ks, buf[:size], cipher)
+    assert torch.equal(cipher, want)
+    cipher = buf[:total].view(torch.int32).view(n, nbits // 32)
+    cipher.copy_(want)
+    back = buf[total // 2:total // 2 + size]
+    ctx.decrypt_message_host(ks, cipher, back, use_crt=True)
+    assert torch.equal(back, msg)
+    ctx.close()
+
+
+@pytest.mark.parametrize("K", [1, 64, 2000])
+def test_pieces_by_key_count_and_priority(K):
+    # 128 chunks a key and piece at least (2,000 keys: one piece), and a stream of another priority.
+    import torch
+
+    import paper_2111_11924_gb300 as P
+
+    nbits, size = 512, 25_000_003
+    ctx = P.Context(0)
+    ks = ctx.keygen(K, nbits, 65537, 34)
+    msg = torch.from_numpy(np.random.default_rng(3).integers(0, 256, size, dtype=np.uint8)).pin_memory()
+    n = P.num_chunks(size, nbits)
+    want = ctx.encrypt_chunks(ks, ctx.split(nbits, msg.cuda())).cpu()
+    for s in (None, torch.cuda.Stream(priority=-1)):
+        cipher = _pinned((n, nbits // 32), torch.int32)
+        ctx.encrypt_message_host(ks, msg, cipher, stream=s)
+        assert torch.equal(cipher, want)
+    ctx.close()
+
+
 def test_errors_in_pieces(monkeypatch):
     import torch
 
