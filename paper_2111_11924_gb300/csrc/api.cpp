@@ -284,18 +284,22 @@ int key_groups_for(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *key_idx, 
   return rc;
 }
 
-// A *_host call in pieces: each piece's copy in, kernels and copy out are
-// queued on one of kPieceStreams streams, so that the copies of one piece run
-// beside the kernels of the others and a piece's last blocks beside the next
-// one's first.  A piece is at least kPieceBytes of message, enough to fill the
-// GPU several times, has kPieceRows chunks a key at least (a block serves one
-// key: the last block of each is part empty), and starts at a multiple of K
-// chunks (chunk t of the message is chunk t - start of the piece under the
-// same key) and of 16 (aligned message bytes).  Host buffers that overlap go
-// in one piece (all input is read before any output is written), and so does
-// a call on a stream of another priority than the pieces' own.  Measured, one piece on one stream against pieces:
-// encrypting 100 MiB at 2048 bits 8.04 and 7.14 ms, 50 MB at 1024 bits 2.29
-// and 1.90; CRT decryption of 25 MB 58.5 and 58.3.
+// Encryption of a host message in pieces: each piece's copy in, kernels and
+// copy out are queued on one of kPieceStreams streams, so that the copies of
+// one piece run beside the kernels of the others and a piece's last blocks
+// beside the next one's first.  A piece is at least kPieceBytes of message,
+// enough to fill the GPU several times, has kPieceRows chunks a key at least
+// (a block serves one key: the last block of each is part empty), and starts
+// at a multiple of K chunks (chunk t of the message is chunk t - start of the
+// piece under the same key) and of 16 (aligned message bytes).  Host buffers
+// that overlap go in one piece (all input is read before any output is
+// written), and so does a call on a stream of another priority than the
+// pieces' own.  Measured, one piece on one stream against pieces: 100 MiB at
+// 2048 bits 8.04 and 7.14 ms, 50 MB at 1024 bits 2.29 and 1.90, 25 MiB at 4096
+// bits 3.79 and 3.61.  Decryption, where the copies are below 2% of the time,
+// stays in one piece: in pieces, 25 MB with CRT 58.5 and 58.3, but 13 MiB full
+// d at 4096 bits 475.8 and 494.7, 50 MiB at 2048 bits and 512 keys 473.5 and
+// 485.5.
 constexpr size_t kPieceBytes = 6u << 20, kPieceRows = 128, kMaxPieces = 8;
 
 // Chunks per piece for a message of n chunks (n itself: one piece).
@@ -916,27 +920,22 @@ int pmk_decrypt_message_host(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t 
   if (!h_msg || !h_cipher) return PMK_EINVAL;
   DeviceGuard g(ctx->device);
   if (!g.ok()) return PMK_ECUDA;
-  const size_t S = ks->nbits / 32, P = pmk_payload_bytes(ks->nbits), words = n_chunks * S;
+  const size_t words = n_chunks * (ks->nbits / 32);
   cudaStream_t st = as_stream(stream);
   int rc = acquire(ctx->msg, msg_len, st);
   if (rc == PMK_OK) rc = acquire(ctx->a, words * 4, st);
   if (rc == PMK_OK) rc = acquire(ctx->b, words * 4, st);
   uint8_t *m = static_cast<uint8_t *>(ctx->msg.ptr);
   uint32_t *c = static_cast<uint32_t *>(ctx->a.ptr), *p = static_cast<uint32_t *>(ctx->b.ptr);
-  const bool split = !overlap(h_msg, msg_len, h_cipher, n_chunks * S * 4);
   bool queued = false;  // a copy from or to the caller's host memory is in flight
-  if (rc == PMK_OK)
-    rc = in_pieces(ctx, split, msg_len, n_chunks, ks->K, st, [&](size_t first, size_t n, cudaStream_t s) -> int {
-      const size_t byte0 = first * P, len = std::min(n * P, msg_len - byte0), w = first * S;
-      queued = true;
-      if (cudaMemcpyAsync(c + w, h_cipher + w, n * S * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) return PMK_ECUDA;
-      if (pmk::fault_injected("after_copy")) return PMK_ECUDA;
-      int r = enqueue_decrypt(ctx, ks, c + w, p + w, n, use_crt, s);
-      if (r == PMK_OK) r = pmk::launch_join(ks->nbits, p + w, n, m + byte0, len, s);
-      if (r == PMK_OK && cudaMemcpyAsync(h_msg + byte0, m + byte0, len, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        r = PMK_ECUDA;
-      return r;
-    });
+  if (rc == PMK_OK) {
+    queued = true;
+    if (cudaMemcpyAsync(c, h_cipher, words * 4, cudaMemcpyHostToDevice, st) != cudaSuccess) rc = PMK_ECUDA;
+  }
+  if (rc == PMK_OK && pmk::fault_injected("after_copy")) rc = PMK_ECUDA;
+  if (rc == PMK_OK) rc = enqueue_decrypt(ctx, ks, c, p, n_chunks, use_crt, st);
+  if (rc == PMK_OK) rc = pmk::launch_join(ks->nbits, p, n_chunks, m, msg_len, st);
+  if (rc == PMK_OK && cudaMemcpyAsync(h_msg, m, msg_len, cudaMemcpyDeviceToHost, st) != cudaSuccess) rc = PMK_ECUDA;
   release(ctx->msg, st);
   release(ctx->a, st);
   release(ctx->b, st);
