@@ -251,10 +251,10 @@ __host__ __device__ constexpr bool ring() {
   return L <= 3 || TPI == 2;
 }
 
-// A modulus N as the products use it: this lane's limbs of N, and for two or
-// more limbs per lane (see PairSum) of f = F, or F - 2^(32 (S - 2)) mod N with
-// ring(), where F = (k N + 1) / 2^64 and k = -N^-1 mod 2^64.  tight: N is so
-// near 2^(32 S) that a product can reach 2N before its last subtraction.
+// A modulus N as the products use it: this lane's limbs of N, and for the form
+// of PairSum of f = F, or F - 2^(32 (S - 2)) mod N with ring(), where
+// F = (k N + 1) / 2^64 and k = -N^-1 mod 2^64.  tight: N is so near 2^(32 S)
+// that a product can reach 2N before its last subtraction.
 template <int L>
 struct Modulus {
   uint32_t n[L], f[L];
@@ -264,8 +264,8 @@ struct Modulus {
 
 // a <- MontMul(a, y) = a y R^-1 mod N.  a: this lane's limbs (any value < R);
 // ys: y's S limbs in shared or global memory (y < N).
-// One row at a time, one add-with-carry chain per lane: the form for one limb
-// per lane (the residues of 128-bit keys), which has no pairs.
+// One row at a time, one add-with-carry chain per lane: the form for four limbs
+// or fewer (see pair_form).
 template <int S, int TPI>
 __device__ __forceinline__ void mont_mul_chain(uint32_t (&a)[S / TPI], const uint32_t *ys, const Modulus<S / TPI> &m,
                                                uint32_t r) {
@@ -617,13 +617,23 @@ struct OddPairSum {
   }
 };
 
+// Whether products of S limbs on TPI lanes take the form of PairSum: not with
+// one limb per lane, which has no pairs, nor at four limbs, where making F and
+// the last two reductions cost more than the rows (256-bit CRT, 1,700 chunks:
+// 72.5 us in pairs and 67.3 by rows; 8 limbs on 2 lanes, 512-bit CRT, 168 in
+// pairs and 183 by rows).
+template <int S, int TPI>
+__host__ __device__ constexpr bool pair_form() {
+  return S / TPI > 1 && S > 4;
+}
+
 template <int S, int TPI>
 __device__ __forceinline__ void make_modulus(Modulus<S / TPI> &m, const uint32_t *N, uint32_t n0, uint32_t r) {
   constexpr int L = S / TPI;
   load_slice_global<L>(m.n, N, r);
   m.k0 = n0;
   m.tight = false;
-  if constexpr (L > 1) {
+  if constexpr (pair_form<S, TPI>()) {
     // -N^-1 mod 2^64 from its low word by one Newton step, in lane 0
     const uint64_t n01 = ((uint64_t)m.n[1] << 32) | m.n[0];
     m.k1 = (uint32_t)(((uint64_t)n0 * (2 + n01 * n0)) >> 32);
@@ -728,7 +738,7 @@ __device__ __forceinline__ void mont_mul_pairs(uint32_t (&a)[S / TPI], const uin
 
 template <int S, int TPI, bool HOT = false>
 __device__ __forceinline__ void mont(uint32_t (&a)[S / TPI], const uint32_t *ys, const Modulus<S / TPI> &m, uint32_t r) {
-  if constexpr (S / TPI > 1) {
+  if constexpr (pair_form<S, TPI>()) {
     mont_mul_pairs<S, TPI, HOT>(a, ys, m, r);
   } else {
     mont_mul_chain<S, TPI>(a, ys, m, r);
