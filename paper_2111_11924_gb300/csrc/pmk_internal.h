@@ -286,7 +286,7 @@ constexpr size_t kDirectMaxJobs = 256;
 }  // namespace pmk
 
 namespace pmk {
-// The streams over which a *_host call spreads the pieces of a long message
+// The streams over which a host encryption spreads the pieces of a long message
 // (made on first use; idle between calls).
 constexpr int kPieceStreams = 3;
 struct PieceStreams {
