@@ -7,8 +7,10 @@
 // the multiplier a step:
 //     for i in 0, 2, .. S-2:  T += a (y_i + 2^32 y_{i+1});  T = (T + q N) / 2^64
 // with q so that T + q N is divisible (how q is found: PairSum), followed by
-// one conditional subtraction, so every product is canonical (< N).  Exponentiation is Algorithm 2's square-and-multiply generalised to a
-// left-to-right sliding window of odd powers (schedules built on the host).
+// one conditional subtraction, so that a product of operands below N is
+// canonical (< N).  Exponentiation is Algorithm 2's square-and-multiply
+// generalised to a left-to-right sliding window of odd powers (schedules built
+// on the host).
 //
 // Cost model on this GPU (measured with row-shaped loops, MAC per clock per SM
 // at 4 / 8 / 16 warps per SM): a wide multiply-add with carry in and out
@@ -689,7 +691,18 @@ __host__ __device__ constexpr int unrolled_steps() {
 }
 
 // a <- MontMul(a, y) = a y R^-1 mod N for two or more limbs per lane.
-// a: any value < R; ys: y's S limbs in shared or global memory (y < N).
+// ys: y's S limbs in shared or global memory.
+//
+// Range.  The steps add Q N with Q < R (1 + d), d = 2.01 / 2^64 (the quotients
+// of F stand for products with k < 2^64, or k + 2^64 with ring()), so
+// T < a y / R + N (1 + d).  For a, y < N that is below 2N, or below 3N when
+// tight, and the result is canonical.  For a in [N, R) T is below N (1 + d) + y:
+// the result is congruent but, with y that close to N and N not tight, can be
+// N or just above, below N (1 + d).  CRT pieces and chunks >= N are such
+// operands; the products that follow see values below N (1 + 2 d), after
+// mod_add, and 5 d < 16 / 2^64 keeps them below 2N, so the next result is
+// canonical again, and so is the last one, with 1.  Whoever looks at a value
+// before that takes N for zero (k_blind_crt).
 //
 // Bound: the wide multiply-add, 4 L per lane and step at 4 clocks of the
 // fma-heavy pipe each, against about 20 other instructions a step (64 limbs
