@@ -1,6 +1,7 @@
 // C ABI of the PMKRSA library (include/pmkrsa.h): argument checks, key-set
 // upload, and the order of kernel launches for each call.
 #include <algorithm>
+#include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <map>
@@ -889,13 +890,16 @@ int pmk_encrypt_message_host(pmk_ctx *ctx, const pmk_keyset *ks, const uint8_t *
   uint32_t *c = static_cast<uint32_t *>(ctx->a.ptr);
   const bool split = !overlap(h_msg, msg_len, h_cipher, n_chunks * S * 4);
   bool queued = false;  // a copy from or to the caller's host memory is in flight
+  int piece = 0;
   if (rc == PMK_OK)
     rc = in_pieces(ctx, split, msg_len, n_chunks, ks->K, st, [&](size_t first, size_t n, cudaStream_t s) -> int {
       const size_t byte0 = first * P, len = std::min(n * P, msg_len - byte0);
       uint32_t *cp = c + first * S;
       queued = true;
       if (cudaMemcpyAsync(m + byte0, h_msg + byte0, len, cudaMemcpyHostToDevice, s) != cudaSuccess) return PMK_ECUDA;
-      if (pmk::fault_injected("after_copy")) return PMK_ECUDA;
+      char site[32];
+      std::snprintf(site, sizeof site, "after_copy:%d", piece++);
+      if (pmk::fault_injected("after_copy") || pmk::fault_injected(site)) return PMK_ECUDA;
       int r = pmk::launch_split(ks->nbits, m + byte0, len, cp, n, s);
       if (r == PMK_OK) r = enqueue_encrypt(ctx, ks, cp, cp, n, s);
       if (r == PMK_OK && cudaMemcpyAsync(h_cipher + first * S, cp, n * S * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess)

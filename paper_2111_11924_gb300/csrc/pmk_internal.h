@@ -59,7 +59,8 @@ constexpr size_t kMaxChunks = (size_t)1 << 32;
 // PMK_INJECT_FAULT names `site`.  The *_host calls consult it right after
 // they queue the copy of the caller's input ("after_copy") and then fail as a
 // failed launch would, so a test can check that an error path leaves no
-// copy of a caller's buffer in flight.  Nothing on the GPU faults.
+// copy of a caller's buffer in flight; "after_copy:i" fails an encryption at
+// its piece i (0 first) only.  Nothing on the GPU faults.
 bool fault_injected(const char *site);
 
 // Exponent schedule for left-to-right sliding-window exponentiation.
