@@ -294,14 +294,34 @@ int key_groups_for(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *key_idx, 
 // at a multiple of K chunks (chunk t of the message is chunk t - start of the
 // piece under the same key) and of 16 (aligned message bytes).  Host buffers
 // that overlap go in one piece (all input is read before any output is
-// written), and so does a call on a stream of another priority than the
-// pieces' own.  Measured, one piece on one stream against pieces: 100 MiB at
-// 2048 bits 8.04 and 7.14 ms, 50 MB at 1024 bits 2.29 and 1.90, 25 MiB at 4096
-// bits 3.79 and 3.61.  Decryption, where the copies are below 2% of the time,
-// stays in one piece: in pieces, 25 MB with CRT 58.5 and 58.3, but 13 MiB full
-// d at 4096 bits 475.8 and 494.7, 50 MiB at 2048 bits and 512 keys 473.5 and
-// 485.5.
+// written), and so does a call whose output is not page-locked, or whose stream
+// has another priority than the pieces' own.
+// Measured with page-locked buffers, one piece on one stream against pieces:
+// 100 MiB at 2048 bits 8.04 and 7.14 ms, 50 MB at 1024 bits 2.29 and 1.90,
+// 25 MiB at 4096 bits 3.79 and 3.61.  Decryption, where the copies are below 2%
+// of the time, stays in one piece: in pieces, 25 MB with CRT 58.5 and 58.3, but
+// 13 MiB full d at 4096 bits 475.8 and 494.7, 50 MiB at 2048 bits and 512 keys
+// 473.5 and 485.5.
 constexpr size_t kPieceBytes = 6u << 20, kPieceRows = 128, kMaxPieces = 8;
+
+// Whether the first and last byte of [p, p + n) are page-locked host memory.
+// A copy to pageable memory returns only when it is done, so pieces would run
+// one after another there, with a part-empty GPU at the end of each: from and
+// to pageable memory, 100 MiB at 2048 bits takes 8.65 ms in pieces and 8.12 in
+// one, at 512 bits 3.52 and 3.24, 50 MB at 1024 bits 2.64 and 2.34.  (A copy
+// from pageable memory is staged and does not hold the pieces up: 7.14 ms for
+// 100 MiB at 2048 bits to page-locked memory, from either kind.)
+bool page_locked(const void *p, size_t n) {
+  for (const char *x : {static_cast<const char *>(p), static_cast<const char *>(p) + n - 1}) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, x) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (a.type != cudaMemoryTypeHost) return false;
+  }
+  return true;
+}
 
 // Chunks per piece for a message of n chunks (n itself: one piece).
 size_t piece_chunks(size_t msg_len, size_t n, uint32_t K) {
@@ -312,13 +332,12 @@ size_t piece_chunks(size_t msg_len, size_t n, uint32_t K) {
   return std::min(n, ((n + pieces - 1) / pieces + unit - 1) / unit * unit);
 }
 
-// queue(first chunk, chunks, stream) for every piece; `split` false asks for
-// one piece.  With one piece that is the caller's stream; else the pieces begin
-// after all that `st` holds, and `st` waits for them all.  On an error the
-// piece streams are idle on return.
+// queue(first chunk, chunks, stream) for every piece of `per` chunks.  With one
+// piece (per = n) that is the caller's stream; else the pieces begin after all
+// that `st` holds, and `st` waits for them all.  On an error the piece streams
+// are idle on return.
 template <typename Queue>
-int in_pieces(pmk_ctx *ctx, bool split, size_t msg_len, size_t n, uint32_t K, cudaStream_t st, Queue queue) {
-  const size_t per = split ? piece_chunks(msg_len, n, K) : n;
+int in_pieces(pmk_ctx *ctx, size_t per, size_t n, cudaStream_t st, Queue queue) {
   int priority = 0;  // the piece streams' own
   if (per < n && cudaStreamGetPriority(st, &priority) != cudaSuccess) return PMK_ECUDA;
   if (per == n || priority != 0) return queue((size_t)0, n, st);
@@ -888,11 +907,14 @@ int pmk_encrypt_message_host(pmk_ctx *ctx, const pmk_keyset *ks, const uint8_t *
   if (rc == PMK_OK) rc = acquire(ctx->a, n_chunks * S * 4, st);
   uint8_t *m = static_cast<uint8_t *>(ctx->msg.ptr);
   uint32_t *c = static_cast<uint32_t *>(ctx->a.ptr);
-  const bool split = !overlap(h_msg, msg_len, h_cipher, n_chunks * S * 4);
+  size_t per = piece_chunks(msg_len, n_chunks, ks->K);
+  if (per < n_chunks &&
+      (overlap(h_msg, msg_len, h_cipher, n_chunks * S * 4) || !page_locked(h_cipher, n_chunks * S * 4)))
+    per = n_chunks;
   bool queued = false;  // a copy from or to the caller's host memory is in flight
   int piece = 0;
   if (rc == PMK_OK)
-    rc = in_pieces(ctx, split, msg_len, n_chunks, ks->K, st, [&](size_t first, size_t n, cudaStream_t s) -> int {
+    rc = in_pieces(ctx, per, n_chunks, st, [&](size_t first, size_t n, cudaStream_t s) -> int {
       const size_t byte0 = first * P, len = std::min(n * P, msg_len - byte0);
       uint32_t *cp = c + first * S;
       queued = true;

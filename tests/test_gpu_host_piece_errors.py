@@ -51,3 +51,20 @@ def test_a_piece_past_the_last_is_not_reached(env, monkeypatch):
     cipher.zero_()
     ctx.encrypt_message_host(ks, msg, cipher)
     assert torch.equal(cipher, want)
+
+
+def test_pageable_output_goes_in_one_piece(env, monkeypatch):
+    """A copy to pageable memory holds the call up, so pieces would run one
+    after another; a pageable input does not matter."""
+    import torch
+
+    P, ctx, ks, msg, cipher, want = env
+    monkeypatch.setenv("PMK_INJECT_FAULT", "after_copy:1")
+    pageable = torch.zeros_like(want)
+    assert not pageable.is_pinned()
+    for src in (msg, msg.clone()):
+        pageable.zero_()
+        ctx.encrypt_message_host(ks, src, pageable)
+        assert torch.equal(pageable, want)
+        with pytest.raises(P.PMKError):
+            ctx.encrypt_message_host(ks, src, cipher)
