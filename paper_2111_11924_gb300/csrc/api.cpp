@@ -7,6 +7,7 @@
 #include <map>
 #include <new>
 
+#include "host_pieces.h"
 #include "pmk_internal.h"
 
 namespace {
@@ -285,25 +286,6 @@ int key_groups_for(pmk_ctx *ctx, const pmk_keyset *ks, const uint32_t *key_idx, 
   return rc;
 }
 
-// Encryption of a host message in pieces: each piece's copy in, kernels and
-// copy out are queued on one of kPieceStreams streams, so that the copies of
-// one piece run beside the kernels of the others and a piece's last blocks
-// beside the next one's first.  A piece is at least kPieceBytes of message,
-// enough to fill the GPU several times, has kPieceRows chunks a key at least
-// (a block serves one key: the last block of each is part empty), and starts
-// at a multiple of K chunks (chunk t of the message is chunk t - start of the
-// piece under the same key) and of 16 (aligned message bytes).  Host buffers
-// that overlap go in one piece (all input is read before any output is
-// written), and so does a call whose output is not page-locked, or whose stream
-// has another priority than the pieces' own.
-// Measured with page-locked buffers, one piece on one stream against pieces:
-// 100 MiB at 2048 bits 8.04 and 7.14 ms, 50 MB at 1024 bits 2.29 and 1.90,
-// 25 MiB at 4096 bits 3.79 and 3.61.  Decryption, where the copies are below 2%
-// of the time, stays in one piece: in pieces, 25 MB with CRT 58.5 and 58.3, but
-// 13 MiB full d at 4096 bits 475.8 and 494.7, 50 MiB at 2048 bits and 512 keys
-// 473.5 and 485.5.
-constexpr size_t kPieceBytes = 6u << 20, kPieceRows = 128, kMaxPieces = 8;
-
 // Whether the first and last byte of [p, p + n) are page-locked host memory.
 // A copy to pageable memory returns only when it is done, so pieces would run
 // one after another there, with a part-empty GPU at the end of each: from and
@@ -321,15 +303,6 @@ bool page_locked(const void *p, size_t n) {
     if (a.type != cudaMemoryTypeHost) return false;
   }
   return true;
-}
-
-// Chunks per piece for a message of n chunks (n itself: one piece).
-size_t piece_chunks(size_t msg_len, size_t n, uint32_t K) {
-  const size_t pieces = std::min({kMaxPieces, msg_len / kPieceBytes, n / (kPieceRows * K)});
-  if (pieces < 2) return n;
-  size_t unit = K;
-  while (unit % 16) unit *= 2;
-  return std::min(n, ((n + pieces - 1) / pieces + unit - 1) / unit * unit);
 }
 
 // queue(first chunk, chunks, stream) for every piece of `per` chunks.  With one
@@ -907,7 +880,7 @@ int pmk_encrypt_message_host(pmk_ctx *ctx, const pmk_keyset *ks, const uint8_t *
   if (rc == PMK_OK) rc = acquire(ctx->a, n_chunks * S * 4, st);
   uint8_t *m = static_cast<uint8_t *>(ctx->msg.ptr);
   uint32_t *c = static_cast<uint32_t *>(ctx->a.ptr);
-  size_t per = piece_chunks(msg_len, n_chunks, ks->K);
+  size_t per = pmk::piece_chunks(msg_len, n_chunks, ks->K);
   if (per < n_chunks &&
       (overlap(h_msg, msg_len, h_cipher, n_chunks * S * 4) || !page_locked(h_cipher, n_chunks * S * 4)))
     per = n_chunks;
