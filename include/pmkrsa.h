@@ -428,8 +428,19 @@ int pmk_measure_imad_peak(pmk_ctx *ctx, double *mad_lo_per_clk_per_sm, double *s
  */
 int pmk_set_kernel_config(pmk_ctx *ctx, uint32_t limbs, int crt, uint32_t tpi, uint32_t form);
 /* The geometry set for (limbs, crt), else the built-in one of calls that fill
- * the GPU (smaller calls may take more lanes).  EINVAL for a NULL argument, EUNSUPPORTED if no kernel is compiled for (limbs, crt). */
+ * the GPU (smaller calls may take more lanes).  EINVAL for a NULL argument,
+ * EUNSUPPORTED if no kernel is compiled for (limbs, crt). */
 int pmk_get_kernel_config(const pmk_ctx *ctx, uint32_t limbs, int crt, uint32_t *tpi, uint32_t *form);
+/* The geometry and window bound that a call of this context on n_chunks chunks
+ * of ks runs (crt = 0: encryption and full-d decryption, 1: CRT decryption):
+ * what is set for that width, else the built-in choice for that many.  EINVAL
+ * for a NULL argument, a key set of another device or n_chunks = 0,
+ * EUNSUPPORTED if no kernel is compiled for the width. */
+int pmk_get_call_config(const pmk_ctx *ctx, const pmk_keyset *ks, int crt, size_t n_chunks, uint32_t *tpi,
+                        uint32_t *form, uint32_t *max_window);
+/* Give dst what src has set for (limbs, crt), geometry and window bound; where
+ * src has nothing set, dst has nothing set either.  EINVAL for a NULL context. */
+int pmk_copy_kernel_config(pmk_ctx *dst, const pmk_ctx *src, uint32_t limbs, int crt);
 /* Compiled geometries for (limbs, crt): writes up to `max` (tpi, form) pairs
  * and returns how many exist (a negative code on bad arguments).  Host only. */
 int pmk_list_kernel_configs(uint32_t limbs, int crt, uint32_t *tpi, uint32_t *form, int max);

@@ -100,6 +100,16 @@ pmk::KernelConfig call_cfg(const pmk_ctx *ctx, const pmk_keyset *ks, bool crt, s
                               ctx->sms);
 }
 
+// dst[key] becomes src[key], or is removed where src has none.
+template <typename Map>
+void copy_entry(Map &dst, const Map &src, uint32_t key) {
+  const auto it = src.find(key);
+  if (it != src.end())
+    dst[key] = it->second;
+  else
+    dst.erase(key);
+}
+
 // Whether any geometry for (limbs, crt) is compiled with the small table.
 bool small_table_available(uint32_t limbs, bool crt) {
   pmk::KernelConfig v[64];
@@ -993,6 +1003,26 @@ int pmk_get_kernel_config(const pmk_ctx *ctx, uint32_t limbs, int crt, uint32_t 
   if (c.tpi == 0) return PMK_EUNSUPPORTED;
   *tpi = c.tpi;
   *form = c.form;
+  return PMK_OK;
+}
+
+int pmk_get_call_config(const pmk_ctx *ctx, const pmk_keyset *ks, int crt, size_t n_chunks, uint32_t *tpi,
+                        uint32_t *form, uint32_t *max_window) {
+  if (!ctx || !ks || ks->device != ctx->device || n_chunks == 0 || !tpi || !form || !max_window) return PMK_EINVAL;
+  const pmk::KernelConfig c = call_cfg(ctx, ks, crt != 0, n_chunks);
+  if (c.tpi == 0) return PMK_EUNSUPPORTED;
+  *tpi = c.tpi;
+  *form = c.form;
+  *max_window = pmk::window_of(c.table);
+  return PMK_OK;
+}
+
+int pmk_copy_kernel_config(pmk_ctx *dst, const pmk_ctx *src, uint32_t limbs, int crt) {
+  if (!dst || !src) return PMK_EINVAL;
+  if (dst == src) return PMK_OK;
+  const uint32_t key = limbs << 1 | (crt ? 1u : 0u);
+  copy_entry(dst->cfg, src->cfg, key);
+  copy_entry(dst->table, src->table, key);
   return PMK_OK;
 }
 

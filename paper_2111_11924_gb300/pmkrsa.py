@@ -89,6 +89,8 @@ def load_library() -> ctypes.CDLL:
                                       ctypes.POINTER(i)]),
         "pmk_set_kernel_config": (i, [vp, u32, i, u32, u32]),
         "pmk_get_kernel_config": (i, [vp, u32, i, P32, P32]),
+        "pmk_get_call_config": (i, [vp, vp, i, sz, P32, P32, P32]),
+        "pmk_copy_kernel_config": (i, [vp, vp, u32, i]),
         "pmk_list_kernel_configs": (i, [u32, i, P32, P32, i]),
         "pmk_set_kernel_window": (i, [vp, u32, i, u32]),
         "pmk_get_kernel_window": (i, [vp, u32, i, P32]),
@@ -538,16 +540,21 @@ class Context:
         return res
 
     def copy_kernel_configs_from(self, other: "Context", keysets: dict) -> None:
-        """Take other's kernel geometry and window bound for every limb count
-        the key sets use (full width and CRT residues).  A width where other
-        has the built-in geometry stays unset, so that each call's size picks
-        its lanes."""
+        """Take what other has set (kernel geometry and window bound) for
+        every limb count the key sets use, full width and CRT residues.  A
+        width for which other has nothing set is unset here too, so that each
+        call's size picks its lanes."""
         for ks in keysets.values():
             for limbs, crt in ((ks.nbits // 32, False), (ks.nbits // 32 // ks.nprimes, True)):
-                cfg = other.get_kernel_config(limbs, crt)
-                if cfg != self.get_kernel_config(limbs, crt):
-                    self.set_kernel_config(limbs, crt, *cfg)
-                self.set_kernel_window(limbs, crt, other.get_kernel_window(limbs, crt))
+                _check(load_library().pmk_copy_kernel_config(self.handle, other.handle, limbs, int(crt)),
+                       "pmk_copy_kernel_config")
+
+    def get_call_config(self, ks: KeySet, crt: bool, n_chunks: int) -> tuple:
+        """(tpi, form, window bound) of a call on n_chunks chunks of ks."""
+        v = np.zeros(3, np.uint32)
+        _check(load_library().pmk_get_call_config(self.handle, ks.handle, int(crt), n_chunks, _p32(v[0:]), _p32(v[1:]),
+                                                  _p32(v[2:])), "pmk_get_call_config")
+        return int(v[0]), int(v[1]), int(v[2])
 
     def get_kernel_config(self, limbs: int, crt: bool) -> tuple:
         tpi, form = np.zeros(1, np.uint32), np.zeros(1, np.uint32)
