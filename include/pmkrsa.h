@@ -441,6 +441,18 @@ int pmk_get_call_config(const pmk_ctx *ctx, const pmk_keyset *ks, int crt, size_
 /* Give dst what src has set for (limbs, crt), geometry and window bound; where
  * src has nothing set, dst has nothing set either.  EINVAL for a NULL context. */
 int pmk_copy_kernel_config(pmk_ctx *dst, const pmk_ctx *src, uint32_t limbs, int crt);
+/* Set a geometry and window bound that were measured as the fastest for calls
+ * on n_chunks chunks of ks (modes as pmk_autotune, which ends with this call).
+ * Unlike those of pmk_set_kernel_config and pmk_set_kernel_window they serve
+ * calls of about that size: all for which the built-in choice by size is the
+ * same as for n_chunks.  Calls of other sizes run the built-in choice; the task
+ * queues of a batch run the geometry set.  pmk_get_kernel_config and
+ * pmk_get_kernel_window report it, and the two setters replace it.  EINVAL for
+ * a NULL argument, a key set of another device, n_chunks = 0, a mode outside
+ * 0..2 or a window bound other than 0, 4 and 5; EUNSUPPORTED if that geometry
+ * or bound is not compiled in. */
+int pmk_set_tuned_config(pmk_ctx *ctx, const pmk_keyset *ks, size_t n_chunks, int mode, uint32_t tpi, uint32_t form,
+                         uint32_t max_window);
 /* Compiled geometries for (limbs, crt): writes up to `max` (tpi, form) pairs
  * and returns how many exist (a negative code on bad arguments).  Host only. */
 int pmk_list_kernel_configs(uint32_t limbs, int crt, uint32_t *tpi, uint32_t *form, int max);
@@ -475,7 +487,7 @@ int pmk_get_kernel_window(const pmk_ctx *ctx, uint32_t limbs, int crt, uint32_t 
  * (mode 0 = encrypt, 1 = full-d decrypt, 2 = CRT decrypt), `reps` timed
  * launches each after one warm-up, and make the fastest the context's
  * geometry and window for that limb count and mode (as
- * pmk_set_kernel_config and pmk_set_kernel_window would).  Writes the
+ * pmk_set_tuned_config would).  Writes the
  * geometry and its best launch time in ms (any output pointer may be NULL);
  * pmk_get_kernel_window reads the window chosen.  Allocates and frees two
  * temporary device buffers and synchronises the device's legacy stream.

@@ -90,14 +90,9 @@ pmk::KernelConfig cfg_for(const pmk_ctx *ctx, uint32_t limbs, bool crt) {
   return c;
 }
 
-// Kernel geometry of a call on n chunks: what the context sets for this width
-// and mode, else the choice for that many exponentiations.
+// Kernel geometry of a call on n chunks.
 pmk::KernelConfig call_cfg(const pmk_ctx *ctx, const pmk_keyset *ks, bool crt, size_t n) {
-  const uint32_t limbs = ks->nbits / 32 / (crt ? ks->nprimes : 1u), key = limbs << 1 | (crt ? 1u : 0u);
-  if (ctx->cfg.count(key) || ctx->table.count(key)) return cfg_for(ctx, limbs, crt);
-  const long long K = ks->K;
-  return pmk::config_for_load(limbs, crt, pmk::Load{K * (crt ? ks->nprimes : 1u), ((long long)n + K - 1) / K, 0},
-                              ctx->sms);
+  return pmk::config_for_call(ctx, ks->nbits / 32 / (crt ? ks->nprimes : 1u), crt, pmk::load_of(ks, crt, n));
 }
 
 // dst[key] becomes src[key], or is removed where src has none.
@@ -355,6 +350,18 @@ void drop(pmk::PieceStreams &p) {
 }  // namespace
 
 namespace pmk {
+KernelConfig config_for_call(const pmk_ctx *ctx, uint32_t limbs, bool crt, const Load &load) {
+  const uint32_t key = limbs << 1 | (crt ? 1u : 0u);
+  if (ctx->cfg.count(key) || ctx->table.count(key)) {
+    const auto t = ctx->tuned.find(key);
+    if (t == ctx->tuned.end()) return cfg_for(ctx, limbs, crt);
+    const KernelConfig here = config_for_load(limbs, crt, load, ctx->sms);
+    if (here.tpi != config_for_load(limbs, crt, t->second, ctx->sms).tpi) return here;
+    return cfg_for(ctx, limbs, crt);
+  }
+  return config_for_load(limbs, crt, load, ctx->sms);
+}
+
 bool fault_injected(const char *site) {
   const char *v = std::getenv("PMK_INJECT_FAULT");
   return v && std::strcmp(v, site) == 0;
@@ -987,13 +994,13 @@ int pmk_measure_imad_peak(pmk_ctx *ctx, double *mad_lo_per_clk_per_sm, double *s
 int pmk_set_kernel_config(pmk_ctx *ctx, uint32_t limbs, int crt, uint32_t tpi, uint32_t form) {
   if (!ctx) return PMK_EINVAL;
   const uint32_t key = limbs << 1 | (crt ? 1u : 0u);
-  if (tpi == 0) {
-    ctx->cfg.erase(key);
-    return PMK_OK;
-  }
   const pmk::KernelConfig c{tpi, form};
-  if (!pmk::modexp_built(limbs, c, crt != 0)) return PMK_EUNSUPPORTED;
-  ctx->cfg[key] = c;
+  if (tpi != 0 && !pmk::modexp_built(limbs, c, crt != 0)) return PMK_EUNSUPPORTED;
+  ctx->tuned.erase(key);
+  if (tpi == 0)
+    ctx->cfg.erase(key);
+  else
+    ctx->cfg[key] = c;
   return PMK_OK;
 }
 
@@ -1004,6 +1011,18 @@ int pmk_get_kernel_config(const pmk_ctx *ctx, uint32_t limbs, int crt, uint32_t 
   *tpi = c.tpi;
   *form = c.form;
   return PMK_OK;
+}
+
+int pmk_set_tuned_config(pmk_ctx *ctx, const pmk_keyset *ks, size_t n_chunks, int mode, uint32_t tpi, uint32_t form,
+                         uint32_t max_window) {
+  if (!ctx || !ks || ks->device != ctx->device || n_chunks == 0 || mode < 0 || mode > 2) return PMK_EINVAL;
+  const bool crt = mode == 2;
+  const uint32_t limbs = ks->nbits / 32 / (crt ? ks->nprimes : 1u);
+  if (!pmk::modexp_built(limbs, pmk::KernelConfig{tpi, form}, crt)) return PMK_EUNSUPPORTED;
+  int rc = pmk_set_kernel_window(ctx, limbs, crt, max_window);
+  if (rc == PMK_OK) rc = pmk_set_kernel_config(ctx, limbs, crt, tpi, form);
+  if (rc == PMK_OK) ctx->tuned[limbs << 1 | (crt ? 1u : 0u)] = pmk::load_of(ks, crt, n_chunks);
+  return rc;
 }
 
 int pmk_get_call_config(const pmk_ctx *ctx, const pmk_keyset *ks, int crt, size_t n_chunks, uint32_t *tpi,
@@ -1023,6 +1042,7 @@ int pmk_copy_kernel_config(pmk_ctx *dst, const pmk_ctx *src, uint32_t limbs, int
   const uint32_t key = limbs << 1 | (crt ? 1u : 0u);
   copy_entry(dst->cfg, src->cfg, key);
   copy_entry(dst->table, src->table, key);
+  copy_entry(dst->tuned, src->tuned, key);
   return PMK_OK;
 }
 
@@ -1032,6 +1052,7 @@ int pmk_set_kernel_window(pmk_ctx *ctx, uint32_t limbs, int crt, uint32_t max_wi
   if (pmk::list_configs(limbs, crt != 0, nullptr, 0) <= 0) return PMK_EUNSUPPORTED;
   if (max_window == pmk::kWindowSmall && !small_table_available(limbs, crt != 0)) return PMK_EUNSUPPORTED;
   const uint32_t key = limbs << 1 | (crt ? 1u : 0u);
+  ctx->tuned.erase(key);
   if (max_window == pmk::kWindowSmall)
     ctx->table[key] = pmk::kTableSmall;
   else

@@ -84,14 +84,12 @@ void arrange_direct(const pmk_ctx *ctx, const std::vector<pmk::PlanJob> &jobs, s
   });
   for (pmk::PlanDirect &d : direct) {
     const pmk::PlanJob &j = jobs[d.job];
-    const uint32_t key = d.limbs << 1 | (is_crt(d) ? 1u : 0u);
-    if (ctx->cfg.count(key) || ctx->table.count(key)) continue;
     double beside = 0;
     for (const pmk::PlanDirect &o : direct)
       if (&o != &d) beside += count(o) * std::min(1.0, length(o) / length(d));
     const long long K = j.K, rows = K * (is_crt(d) ? j.nprimes : 1u);
-    d.cfg = pmk::config_for_load(d.limbs, is_crt(d),
-                                 pmk::Load{rows, ((long long)j.n_chunks + K - 1) / K, (long long)beside}, ctx->sms);
+    d.cfg = pmk::config_for_call(ctx, d.limbs, is_crt(d),
+                                 pmk::Load{rows, ((long long)j.n_chunks + K - 1) / K, (long long)beside});
   }
 }
 

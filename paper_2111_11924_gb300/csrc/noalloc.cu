@@ -102,13 +102,12 @@ extern "C" int pmk_decrypt_message_host_noalloc(const pmk_keyset *ks, const uint
       rc = PMK_ECUDA;
       break;
     }
-    const long long K = ks->K, per_key = ((long long)n_chunks + K - 1) / K;
     if (use_crt) rc = launch_range_check(ks->d_keys, ks->K, S, d_cipher, n_chunks, d_status, st);
     if (!use_crt)
-      rc = launch_modexp(ExpMode::kDecrypt, S, config_for_load(S, false, Load{K, per_key, 0}, sms), ks->d_keys, ks->K,
+      rc = launch_modexp(ExpMode::kDecrypt, S, config_for_load(S, false, load_of(ks, false, n_chunks), sms), ks->d_keys, ks->K,
                          d_cipher, d_plain, n_chunks, st, B, nullptr, kGroupAlign, d_status);
     if (rc == PMK_OK && use_crt) {
-      rc = launch_modexp(ExpMode::kCrtHalf, H, config_for_load(H, true, Load{K * B, per_key, 0}, sms), ks->d_keys, ks->K,
+      rc = launch_modexp(ExpMode::kCrtHalf, H, config_for_load(H, true, load_of(ks, true, n_chunks), sms), ks->d_keys, ks->K,
                          d_cipher, d_plain, n_chunks, st, B);
       if (rc == PMK_OK)
         rc = launch_crt_sum(S, B, ks->d_keys, ks->K, d_plain, n_chunks, st);

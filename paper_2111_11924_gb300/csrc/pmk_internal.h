@@ -269,6 +269,12 @@ struct pmk_keyset {
 };
 
 namespace pmk {
+// A call on n chunks of ks (all primes of each with crt), nothing beside it.
+inline Load load_of(const pmk_keyset *ks, bool crt, size_t n) {
+  const long long K = ks->K;
+  return Load{K * (crt ? ks->nprimes : 1u), ((long long)n + K - 1) / K, 0};
+}
+
 // A grow-only device buffer owned by a context, allocated and freed in
 // stream order (cudaMallocAsync / cudaFreeAsync).  `last_use` is recorded
 // on the stream of the last call that used it; the next call waits on it on
@@ -306,5 +312,15 @@ struct pmk_ctx {
   pmk::PieceStreams pieces;
   std::map<uint32_t, pmk::KernelConfig> cfg;  // (limbs << 1 | crt) -> kernel geometry override
   std::map<uint32_t, int> table;              // (limbs << 1 | crt) -> odd-power table size override
+  std::map<uint32_t, pmk::Load> tuned;        // (limbs << 1 | crt) -> the load at which the tuner chose them
   size_t batch_direct_max = pmk::kDirectMaxJobs;  // pmk_set_batch_direct_max
 };
+
+namespace pmk {
+// Geometry of a call with that load: what the context sets for this width and
+// mode, else the built-in choice by load.  A tuned geometry holds where that
+// choice is the one it was at the tuned load.  (Tuned at 4,113 chunks and held
+// at every size, full d at 2048 bits took 7.98 ms for 403 chunks, 2.95 by
+// load; CRT 2.21 and 0.99; at 1024 bits full d 2.20 and 0.95.)
+KernelConfig config_for_call(const pmk_ctx *ctx, uint32_t limbs, bool crt, const Load &load);
+}  // namespace pmk

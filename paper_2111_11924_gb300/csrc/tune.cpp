@@ -74,8 +74,7 @@ extern "C" int pmk_autotune(pmk_ctx *ctx, const pmk_keyset *ks, size_t n_chunks,
   cudaFree(d_in);
   cudaFree(d_out);
   if (rc == PMK_OK) {
-    rc = pmk_set_kernel_config(ctx, limbs, crt ? 1 : 0, best.tpi, best.form);
-    if (rc == PMK_OK) rc = pmk_set_kernel_window(ctx, limbs, crt ? 1 : 0, pmk::window_of(best.table));
+    rc = pmk_set_tuned_config(ctx, ks, n_chunks, mode, best.tpi, best.form, pmk::window_of(best.table));
     if (tpi) *tpi = best.tpi;
     if (form) *form = best.form;
     if (ms) *ms = best_ms;

@@ -90,6 +90,7 @@ def load_library() -> ctypes.CDLL:
         "pmk_set_kernel_config": (i, [vp, u32, i, u32, u32]),
         "pmk_get_kernel_config": (i, [vp, u32, i, P32, P32]),
         "pmk_get_call_config": (i, [vp, vp, i, sz, P32, P32, P32]),
+        "pmk_set_tuned_config": (i, [vp, vp, sz, i, u32, u32, u32]),
         "pmk_copy_kernel_config": (i, [vp, vp, u32, i]),
         "pmk_list_kernel_configs": (i, [u32, i, P32, P32, i]),
         "pmk_set_kernel_window": (i, [vp, u32, i, u32]),
@@ -516,10 +517,11 @@ class Context:
     def autotune(self, ks: KeySet, n_chunks: int, mode: str = "decrypt", reps: int = 3,
                  cache: "TuneCache | None" = None) -> dict:
         """Time every compiled geometry, with each window bound (5 and 4), for
-        this key set and batch size; keep the fastest.  mode: "encrypt",
-        "decrypt" (full d) or "crt".  With a TuneCache, a result stored for
-        this GPU, width, prime count, mode and batch-size bucket is applied
-        without timing, and a new result is stored."""
+        this key set and batch size; keep the fastest for calls of about that
+        size.  mode: "encrypt", "decrypt" (full d) or "crt".  With a
+        TuneCache, a result stored for this GPU, width, prime count, mode and
+        batch-size bucket is applied without timing, and a new result is
+        stored."""
         m = {"encrypt": 0, "decrypt": 1, "crt": 2}[mode]
         limbs = ks.nbits // 32 // (ks.nprimes if mode == "crt" else 1)
         key = None
@@ -527,8 +529,7 @@ class Context:
             key = cache.key(_torch().cuda.get_device_name(self.device), ks.nbits, ks.nprimes, mode, n_chunks)
             hit = cache.get(key)
             if hit is not None:
-                self.set_kernel_config(limbs, mode == "crt", hit["tpi"], hit["form"])
-                self.set_kernel_window(limbs, mode == "crt", hit["window"])
+                self.set_tuned_config(ks, n_chunks, mode, hit["tpi"], hit["form"], hit["window"])
                 return dict(hit) | {"cached": True}
         tpi, form, ms = np.zeros(1, np.uint32), np.zeros(1, np.uint32), ctypes.c_float()
         _check(load_library().pmk_autotune(self.handle, ks.handle, n_chunks, m, reps, _p32(tpi), _p32(form),
@@ -538,6 +539,13 @@ class Context:
         if cache is not None:
             cache.put(key, res)
         return res
+
+    def set_tuned_config(self, ks: KeySet, n_chunks: int, mode: str, tpi: int, form: int, window: int) -> None:
+        """Set what was measured as the fastest for calls on n_chunks chunks of
+        ks; calls of other sizes keep the built-in choice (pmk_set_tuned_config)."""
+        m = {"encrypt": 0, "decrypt": 1, "crt": 2}[mode]
+        _check(load_library().pmk_set_tuned_config(self.handle, ks.handle, n_chunks, m, tpi, form, window),
+               "pmk_set_tuned_config")
 
     def copy_kernel_configs_from(self, other: "Context", keysets: dict) -> None:
         """Take what other has set (kernel geometry and window bound) for
