@@ -441,6 +441,9 @@ int pmk_get_call_config(const pmk_ctx *ctx, const pmk_keyset *ks, int crt, size_
 /* Give dst what src has set for (limbs, crt), geometry and window bound; where
  * src has nothing set, dst has nothing set either.  EINVAL for a NULL context. */
 int pmk_copy_kernel_config(pmk_ctx *dst, const pmk_ctx *src, uint32_t limbs, int crt);
+/* An identifier of the kernels of this build: results of the tuner that are
+ * kept across processes hold only while it is the same. */
+const char *pmk_kernels_id(void);
 /* Set a geometry and window bound that were measured as the fastest for calls
  * on n_chunks chunks of ks (modes as pmk_autotune, which ends with this call).
  * Unlike those of pmk_set_kernel_config and pmk_set_kernel_window they serve

@@ -6,6 +6,7 @@ against the shared CUDA runtime (the one torch already loaded).
 """
 from __future__ import annotations
 
+import hashlib
 import os
 import shutil
 import subprocess
@@ -40,12 +41,23 @@ def up_to_date() -> bool:
     return all(os.path.getmtime(f) <= t for f in _inputs())
 
 
+def kernels_id(defines: tuple = ()) -> str:
+    """Digest of the sources that decide how fast a geometry runs (kernels and
+    their launch code), for pmk_kernels_id."""
+    h = hashlib.sha256(repr(defines).encode())
+    for f in sorted(os.listdir(CSRC)):
+        if f.endswith((".cu", ".cuh")) or f == "pmk_internal.h":
+            with open(os.path.join(CSRC, f), "rb") as src:
+                h.update(f.encode() + b"\0" + src.read())
+    return h.hexdigest()[:16]
+
+
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False, out: str | None = None,
           defines: tuple = ()) -> str:
     """Compile and link libpmkrsa.so unless it is newer than every source.
 
-    ``out``/``defines`` build a variant elsewhere (for example another row
-    form, ``PMK_ROW_FORM=1``) without touching the in-tree library."""
+    ``out``/``defines`` build a variant elsewhere, with macros of its own,
+    without touching the in-tree library."""
     lib = out or LIB
     if not force and out is None and up_to_date():
         return LIB
@@ -53,7 +65,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False, 
     os.makedirs(obj_dir, exist_ok=True)
     nvcc = _nvcc()
     common = ARCH + ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
-    common += [f"-D{d}" for d in defines]
+    common += [f"-D{d}" for d in (*defines, f'PMK_KERNELS_ID="{kernels_id(defines)}"')]
 
     def compile_one(src: str) -> str:
         obj = os.path.join(obj_dir, src + ".o")

@@ -1046,6 +1046,8 @@ int pmk_copy_kernel_config(pmk_ctx *dst, const pmk_ctx *src, uint32_t limbs, int
   return PMK_OK;
 }
 
+const char *pmk_kernels_id(void) { return PMK_KERNELS_ID; }
+
 int pmk_set_kernel_window(pmk_ctx *ctx, uint32_t limbs, int crt, uint32_t max_window) {
   if (!ctx || (max_window != 0 && max_window != pmk::kWindowFull && max_window != pmk::kWindowSmall))
     return PMK_EINVAL;

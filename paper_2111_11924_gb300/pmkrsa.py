@@ -92,6 +92,7 @@ def load_library() -> ctypes.CDLL:
         "pmk_get_call_config": (i, [vp, vp, i, sz, P32, P32, P32]),
         "pmk_set_tuned_config": (i, [vp, vp, sz, i, u32, u32, u32]),
         "pmk_copy_kernel_config": (i, [vp, vp, u32, i]),
+        "pmk_kernels_id": (ctypes.c_char_p, []),
         "pmk_list_kernel_configs": (i, [u32, i, P32, P32, i]),
         "pmk_set_kernel_window": (i, [vp, u32, i, u32]),
         "pmk_get_kernel_window": (i, [vp, u32, i, P32]),
@@ -574,7 +575,9 @@ class Context:
 class TuneCache:
     """Autotuner results persisted as JSON, keyed by GPU name, key width,
     prime count, mode and batch size rounded up to a power of two (the best
-    geometry depends on how many exponentiations fill the GPU)."""
+    geometry depends on how many exponentiations fill the GPU).  An entry
+    carries the identifier of the kernels it was measured on and is a miss
+    under any others, as is one without."""
 
     def __init__(self, path: str):
         import json
@@ -595,13 +598,13 @@ class TuneCache:
 
     def get(self, key: str):
         e = self.entries.get(key)
-        if e is None:
+        if e is None or e.get("kernels") != load_library().pmk_kernels_id().decode():
             return None
         return {"tpi": int(e["tpi"]), "form": int(e["form"]), "window": int(e.get("window", 5)), "ms": float(e["ms"])}
 
     def put(self, key: str, res: dict) -> None:
         self.entries[key] = {"tpi": int(res["tpi"]), "form": int(res["form"]), "window": int(res.get("window", 5)),
-                             "ms": float(res["ms"])}
+                             "ms": float(res["ms"]), "kernels": load_library().pmk_kernels_id().decode()}
         tmp = f"{self.path}.tmp{self._os.getpid()}"
         with open(tmp, "w") as f:
             self._json.dump(self.entries, f, indent=1, sort_keys=True)
