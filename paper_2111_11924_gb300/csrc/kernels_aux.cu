@@ -342,7 +342,8 @@ const std::vector<ModexpEntry> &built(bool crt) {
 
 const ModexpEntry *find_exact(uint32_t limbs, KernelConfig cfg, bool crt) {
   for (const ModexpEntry &e : built(crt))
-    if (e.limbs == (int)limbs && e.tpi == (int)cfg.tpi && cfg.form < 2 && (e.forms >> cfg.form & 1u) && e.table == cfg.table)
+    if (e.limbs == (int)limbs && e.tpi == (int)cfg.tpi && e.table == cfg.table && cfg.form < 2 &&
+        (e.forms >> cfg.form & 1u))
       return &e;
   return nullptr;
 }
@@ -557,8 +558,9 @@ long long product_clocks(int limbs, int tpi, const Load &load, int sms) {
 // while the GPU has schedulers to spare.  Measured, ms by lanes: full d at
 // 2048 bits, 403 chunks 7.95 (8 lanes) / 4.43 (16) / 2.95 (32), 2,056 chunks
 // 7.95 / 6.38 / 7.77, 4,113 chunks 11.4 / 12.3 / 13.1; CRT at 3072 bits, 685
-// chunks 3.66 (8) / 3.31 (16), 6,000 chunks 12.6 / 14.7.  Fewer lanes than the default are not considered: their tables
-// leave too few exponentiations on an SM.
+// chunks 3.66 (8) / 3.31 (16), 6,000 chunks 12.6 / 14.7.  Fewer lanes than the
+// default are not considered: their tables leave too few exponentiations on an
+// SM.
 KernelConfig config_for_load(uint32_t limbs, bool crt, const Load &load, int sms) {
   KernelConfig best = default_config(limbs, crt);
   if (best.tpi == 0 || sms <= 0) return best;

@@ -266,8 +266,8 @@ struct Modulus {
 
 // a <- MontMul(a, y) = a y R^-1 mod N.  a: this lane's limbs (any value < R);
 // ys: y's S limbs in shared or global memory (y < N).
-// One row at a time, one add-with-carry chain per lane: the form for four limbs
-// or fewer (see pair_form).
+// One row at a time, one add-with-carry chain per lane: the form for one limb
+// per lane and for four limbs on two (see pair_form).
 template <int S, int TPI>
 __device__ __forceinline__ void mont_mul_chain(uint32_t (&a)[S / TPI], const uint32_t *ys, const Modulus<S / TPI> &m,
                                                uint32_t r) {
@@ -353,8 +353,12 @@ __device__ __forceinline__ void mul_wide(uint32_t &lo, uint32_t &hi, uint32_t a,
 // times y_i and the odd limbs times y_{i+1} land on e's pairs, the other two
 // products on o's, so each of the four is one carry chain of L / 2 wide
 // multiply-adds, and T / 2^64 moves whole pairs: e and o keep their roles.
+// (Separate sums for even and odd products are common practice; their spread
+// over lanes, the order of the chains and the ring are this library's own.)
 //
-// Reduction.  F = (k N + 1) / 2^64 with k = -N^-1 mod 2^64 makes
+// Reduction (quotients by Orup 1995, "Simplifying quotient determination in
+// high-radix modular multiplication").  F = (k N + 1) / 2^64 with
+// k = -N^-1 mod 2^64 makes
 // k N = F 2^64 - 1, so adding T mod 2^64 times k N clears the low 64 bits:
 //     T <- floor(T / 2^64) + (T mod 2^64) F.
 // The quotient is lane 0's two low words as they stand, with no product by k
@@ -497,23 +501,18 @@ struct PairSum {
   }
 };
 
-// PairSum for an odd number of limbs per lane (3 or more).  The even limbs are
-// one more than the odd ones, so e ends in weight L and o in weight L + 1, and
-// the words that hold only carries are others: the chains' order differs.
+// PairSum for an odd number of limbs per lane: three, always with ring().  The
+// even limbs are one more than the odd ones, so e ends in weight L and o in
+// weight L + 1, and the words that hold only carries are others: the chains'
+// order differs.
 template <int L, int TPI>
 struct OddPairSum {
+  static_assert(L % 2 == 1 && L > 1 && ring<L, TPI>(), "every lane takes the words of the next one");
   uint32_t e[L + 1], o[L + 1], c1, c2;  // c1, c2: weights 2^(32 (L + 1)), 2^(32 (L + 2))
   uint32_t x0, x1, q0, q1;
-  int above;
-  uint32_t keep;                // zero in the top lane, unless ring()
+  int above;  // the lane above; lane 0 for the top lane
 
-  __device__ __forceinline__ explicit OddPairSum(uint32_t r)
-      : above((int)((r + 1) % TPI)), keep(!ring<L, TPI>() && r == TPI - 1 ? 0u : kFull) {}
-
-  __device__ __forceinline__ uint32_t from_above(uint32_t x) const {
-    return ring<L, TPI>() ? __shfl_sync(kFull, x, above, TPI) : __shfl_down_sync(kFull, x, 1, TPI);
-  }
-  __device__ __forceinline__ uint32_t in(uint32_t x) const { return ring<L, TPI>() ? x : x & keep; }
+  __device__ __forceinline__ explicit OddPairSum(uint32_t r) : above((int)((r + 1) % TPI)) {}
 
   template <bool QUOTIENT>
   __device__ __forceinline__ void send() {
@@ -523,8 +522,8 @@ struct OddPairSum {
       q0 = __shfl_sync(kFull, x0, 0, TPI);
       q1 = __shfl_sync(kFull, x1, 0, TPI);
     }
-    x0 = from_above(x0);
-    x1 = from_above(x1);
+    x0 = __shfl_sync(kFull, x0, above, TPI);
+    x1 = __shfl_sync(kFull, x1, above, TPI);
   }
 
   __device__ __forceinline__ void start(const uint32_t (&a)[L], uint32_t y0, uint32_t y1) {
@@ -555,8 +554,8 @@ struct OddPairSum {
     e[L] = c2;
     pair_chain<L, 0, 0>(e, a, y0);
     addc(d, 0u, 0u);
-    add_cc(e[L - 2], e[L - 2], in(x0));
-    addc_cc(e[L - 1], e[L - 1], in(x1));
+    add_cc(e[L - 2], e[L - 2], x0);
+    addc_cc(e[L - 1], e[L - 1], x1);
     addc_cc(e[L], e[L], 0u);
     addc(d, d, 0u);
     if constexpr (REDUCE) {
@@ -606,8 +605,8 @@ struct OddPairSum {
 
   __device__ __forceinline__ uint32_t shift_out(uint32_t (&t)[L]) {
     uint32_t drop, c;
-    add_cc(e[L], e[L], in(x0));
-    addc_cc(o[L], o[L], in(x1));
+    add_cc(e[L], e[L], x0);
+    addc_cc(o[L], o[L], x1);
     addc(c, c2, 0u);
     add_cc(o[L], o[L], c1);
     addc(c, c, 0u);
@@ -775,8 +774,9 @@ __device__ __forceinline__ void mod_add(uint32_t (&a)[L], const uint32_t (&b)[L]
 // form; on exit a = MontMul(x^E in Montgomery form, last), that is, for any
 // x < N, x^E R^-E last mod N.  tbl: the instance's odd-power table (at least
 // maxidx + 1 rows: the table size the schedule was built for), ybuf: one row
-// of this instance.  sched: steps of make_schedule() (warp-uniform).  Squarings and multiplications share one product in the
-// code, so that it can be unrolled whole.
+// of this instance.  sched: steps of make_schedule() (warp-uniform).
+// Squarings and multiplications share one product in the code, so that it can
+// be unrolled whole.
 template <int S, int TPI>
 __device__ __forceinline__ void exp_window(uint32_t (&a)[S / TPI], uint32_t *tbl, uint32_t *ybuf,
                                            const uint32_t *__restrict__ sched, uint32_t nsteps, uint32_t maxidx,

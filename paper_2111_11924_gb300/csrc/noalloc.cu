@@ -104,11 +104,11 @@ extern "C" int pmk_decrypt_message_host_noalloc(const pmk_keyset *ks, const uint
     }
     if (use_crt) rc = launch_range_check(ks->d_keys, ks->K, S, d_cipher, n_chunks, d_status, st);
     if (!use_crt)
-      rc = launch_modexp(ExpMode::kDecrypt, S, config_for_load(S, false, load_of(ks, false, n_chunks), sms), ks->d_keys, ks->K,
-                         d_cipher, d_plain, n_chunks, st, B, nullptr, kGroupAlign, d_status);
+      rc = launch_modexp(ExpMode::kDecrypt, S, config_for_load(S, false, load_of(ks, false, n_chunks), sms),
+                         ks->d_keys, ks->K, d_cipher, d_plain, n_chunks, st, B, nullptr, kGroupAlign, d_status);
     if (rc == PMK_OK && use_crt) {
-      rc = launch_modexp(ExpMode::kCrtHalf, H, config_for_load(H, true, load_of(ks, true, n_chunks), sms), ks->d_keys, ks->K,
-                         d_cipher, d_plain, n_chunks, st, B);
+      rc = launch_modexp(ExpMode::kCrtHalf, H, config_for_load(H, true, load_of(ks, true, n_chunks), sms),
+                         ks->d_keys, ks->K, d_cipher, d_plain, n_chunks, st, B);
       if (rc == PMK_OK)
         rc = launch_crt_sum(S, B, ks->d_keys, ks->K, d_plain, n_chunks, st);
     }
