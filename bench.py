@@ -55,8 +55,8 @@ KERNELS_PER_STEP = 4  # split, modexp (encrypt), modexp (decrypt), join
 # their own).
 TRAFFIC_SOURCES = ["paper_2111_11924_gb300/csrc/modexp_core.cuh", "paper_2111_11924_gb300/csrc/modexp_grid.cuh"]
 COUNTERS_MEASURED = {  # source digest -> counters of one launch
-    "0eca7bb5e59c25e8": {"traffic": 1140992, "issue_active_pct": 32.88, "warps_active_per_sm": 6.99,
-                         "alu_pipe_pct": 18.94, "fmaheavy_pipe_pct": 77.77, "warp_instructions": 4223030943},
+    "6fa02748bcc4bcd3": {"traffic": 1150208, "issue_active_pct": 32.88, "warps_active_per_sm": 6.99,
+                         "alu_pipe_pct": 18.95, "fmaheavy_pipe_pct": 77.79, "warp_instructions": 4223030943},
 }
 
 
@@ -691,8 +691,9 @@ def batched_leg(ctx, scale: float, reps: int, tune_chunks: int) -> dict:
     Times the plain path (one call, one launch per job, on one stream)
     against the batched path (pmk_batch: one grid launch per job on
     concurrent streams, graph-replayed), after autotuning every
-    (width, mode) on up to tune_chunks chunks, and checks both give
-    identical output."""
+    (width, mode) on up to tune_chunks chunks (which sets the geometry of
+    calls of about that size; the others run the choice by size), and checks
+    both give identical output."""
     import torch
 
     from paper_2111_11924_gb300 import pmkrsa as B

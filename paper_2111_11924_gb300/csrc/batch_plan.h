@@ -39,15 +39,15 @@ struct PlanDirect {
 // of pmk_*_chunks, on a stream of its own) instead of sharing a persistent
 // queue:
 //   - every job, when the batch holds at most kDirectMaxJobs jobs with
-//     chunks: the grid kernel runs each exponentiation faster than the
-//     persistent one (up to 20% on jobs too small to fill the GPU), and the
-//     concurrent launches overlap as well as the shared queue does (mixed
-//     64-message batch 535 vs 552 ms, 256 jobs of 1-16 chunks 61.8 vs
-//     63.8 ms);
+//     chunks: the grid kernel runs with the lanes that suit the job and the
+//     concurrent launches overlap as well as the shared queue does (64 jobs of
+//     16-128 chunks 24.5 against 29.0 ms, 256 jobs of 1-16 chunks 20.2 against
+//     26.9; full d, 1024 to 3072 bits);
 //   - in larger batches, the jobs with at least kDirectWaves GPU-fulls of
-//     exponentiations: one launch per tiny job leaves most of each block's
-//     shared memory unused, and 1,024 jobs of 1-8 chunks took 171 ms as
-//     launches against 94 ms through the queues.
+//     exponentiations: 1,024 jobs of 1-8 chunks took 63.9 ms as launches and
+//     55.3 through the queues (but 28.9 and 41.8 where half of them are CRT
+//     decryptions and a quarter encryptions; the limit was set on earlier
+//     kernels, 171 against 94).
 // (kDirectMaxJobs, the default limit, is defined with the context in
 // pmk_internal.h.)
 constexpr long long kDirectWaves = 1;

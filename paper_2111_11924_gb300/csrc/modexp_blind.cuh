@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(NT, 1) k_blind_crt(const KeyDev *__restrict__ 
   store_slice<L>(tbl, a, r);
   crt_input<S, TPI>(a, cr + t * W, active, parts, sR2, sR3, m, r);     // B = c_r R mod r_i
   // B = 0 mod r_i: crt_input can leave r_i itself (mont_mul_pairs).  Reducing
-  // the pieces first instead took 3,774 and not 3,729 us (2048 bits, 1 MiB).
+  // the pieces first instead took 3,770 and not 3,729 us (2048 bits, 1 MiB).
   uint32_t any = 0, other = 0;  // not 0, not r_i
 #pragma unroll
   for (int j = 0; j < L; j++) {
